@@ -87,6 +87,7 @@ typedef enum {
     PP_Q_BETA = 0, PP_Q_COUT = 1, PP_Q_CIN_G = 2, PP_Q_GROUPS = 3, PP_Q_STRIDE = 4,
     PP_Q_N_GROUPS = 5, PP_Q_N_PATTERNS = 6, PP_Q_IMAGE_BYTES = 7,
     PP_Q_FAST_PATH = 8,       /* 1 if the library equals pp_default_patterns (compiled bodies)  */
+    PP_Q_TENSOR_BYTES = 9,    /* device bytes pp_bind_tensor needs (0: not offered)               */
     PP_Q_SECTION_BYTES = 16   /* + section id: byte size of that section                      */
 } pp_query_key;
 
@@ -140,12 +141,24 @@ int pp_export(pp_handle h, int section, void* host_dst, size_t bytes);
  * Errors: PP_ERR_NULL, PP_ERR_BUFFER (too small), PP_ERR_ALIGN, PP_ERR_CUDA. */
 int pp_bind_device(pp_handle h, void* dev_image, size_t bytes, void* stream);
 
+/* Offer the layer the tensor cores: build its tensor-core weights (every kept weight as a pair of
+ * fp16 values with a common power of two, zeros at the pruned taps; PP_Q_TENSOR_BYTES bytes) in
+ * caller-owned DEVICE memory `dev` (256-byte aligned) from the device image bound before, enqueued
+ * on `stream`.  The same rules as for the image: the caller keeps the memory alive and unmodified
+ * while the handle is used and orders this call before the first pp_conv.  Later calls of pp_conv
+ * and its variants then take the tensor-core kernel wherever it is the faster one; results agree
+ * to fp32 rounding.  Without this call they run on the CUDA cores.  pp_bind_device withdraws it.
+ * Errors: PP_ERR_NULL, PP_ERR_NOT_BOUND, PP_ERR_PATH (PP_Q_TENSOR_BYTES is 0: depthwise layers and
+ * weights of extreme range), PP_ERR_BUFFER (too small), PP_ERR_ALIGN, PP_ERR_CUDA. */
+int pp_bind_tensor(pp_handle h, void* dev, size_t bytes, void* stream);
+
 /* y = sigma(conv3x3(x, W_hat, stride, pad 1) + bias) on the GPU, enqueued on `stream`.
  *   x     DEVICE [N][Cin][H][W] of `dtype` (PP_F32 or PP_F16);
  *   y     DEVICE [N][Cout][Ho][Wo] of the same dtype, Ho = (H-1)/stride + 1 (likewise Wo);
  *         must not overlap x;
  *   bias  DEVICE fp32 [Cout] or NULL (no bias);  relu 0 or 1.
- * Accumulation is fp32 (FFMA on the CUDA cores) in input-channel order; fp16 inputs are
+ * Accumulation is fp32, on the CUDA cores in input-channel order, or on the tensor cores where the
+ * layer is bound for them (pp_bind_tensor); fp16 inputs are
  * widened exactly and the fp16 output is rounded to nearest even.  Pointers need only element
  * alignment; 16-byte aligned x/y with W % 4 == 0 take the vector paths.  N == 0 is a no-op.
  * Validation errors return before any launch; a failed launch returns PP_ERR_CUDA.  Never
@@ -233,6 +246,16 @@ int pp_conv_pool_plan(pp_handle h, int N, int H, int W, size_t workspace_bytes, 
  * of pp_conv_plan.  Host-only. */
 int pp_conv_plan_dt(pp_handle h, int dtype, int pool, int N, int H, int W, size_t workspace_bytes,
                     int64_t* info, int n_info);
+
+/* Whether a call of a layer bound with pp_bind_tensor takes the tensor-core kernel, and how:
+ * info[0] = 1 if so (else 0 and zeros), [1] input-channel splits, [2] workspace bytes used, [3] work
+ * units (pairs of position tiles x filter chunks x splits), [4] positions of a tile, [5] filters of a
+ * unit, [6] and [7] width and height of a tile that is a rectangle of outputs (0: consecutive
+ * positions of the whole batch).  Calls that do not take it run the plan of pp_conv_plan_dt, as all
+ * calls of a layer without pp_bind_tensor do; the workspace to pass is that plan's in either case.
+ * Writes min(n_info, 8) values.  Errors as pp_conv_plan_dt.  Host-only. */
+int pp_conv_tensor_plan(pp_handle h, int dtype, int pool, int N, int H, int W, size_t workspace_bytes,
+                        int64_t* info, int n_info);
 
 /* pp_conv_ws for callers that cannot allocate device memory (the paper has no counterpart to
  * this entry point).  Some callers are not allowed to call cudaMalloc or any allocating routine:

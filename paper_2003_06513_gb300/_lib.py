@@ -22,6 +22,7 @@ SIGNATURES = {
     "pp_query": (_c_int, [_c_void_p, _c_int, ctypes.POINTER(ctypes.c_int64)]),
     "pp_export": (_c_int, [_c_void_p, _c_int, _c_void_p, _c_size_t]),
     "pp_bind_device": (_c_int, [_c_void_p, _c_void_p, _c_size_t, _c_void_p]),
+    "pp_bind_tensor": (_c_int, [_c_void_p, _c_void_p, _c_size_t, _c_void_p]),
     "pp_conv": (_c_int, [_c_void_p, _c_void_p, _c_int, _c_int, _c_int, _c_int, _c_void_p, _c_int,
                          _c_void_p, _c_void_p]),
     "pp_conv_ws": (_c_int, [_c_void_p, _c_void_p, _c_int, _c_int, _c_int, _c_int, _c_void_p, _c_int,
@@ -37,6 +38,8 @@ SIGNATURES = {
                                    ctypes.POINTER(ctypes.c_int64), _c_int]),
     "pp_conv_plan_dt": (_c_int, [_c_void_p, _c_int, _c_int, _c_int, _c_int, _c_int, _c_size_t,
                                  ctypes.POINTER(ctypes.c_int64), _c_int]),
+    "pp_conv_tensor_plan": (_c_int, [_c_void_p, _c_int, _c_int, _c_int, _c_int, _c_int, _c_size_t,
+                                     ctypes.POINTER(ctypes.c_int64), _c_int]),
     "pp_conv_static_scratch": (_c_int, [_c_void_p, _c_void_p, _c_int, _c_int, _c_int, _c_int, _c_void_p,
                                         _c_int, _c_void_p, _c_void_p]),
     "pp_static_scratch_bytes": (_c_int, [ctypes.POINTER(_c_size_t)]),

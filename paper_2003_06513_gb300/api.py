@@ -21,7 +21,7 @@ SECTIONS = {"header": 0, "pid": 1, "perm": 2, "desc": 3, "kofs": 4, "vals": 5, "
 SECTION_DTYPES = {"header": np.uint32, "pid": np.int8, "perm": np.uint32, "desc": np.uint64,
                   "kofs": np.uint32, "vals": np.float32, "dense": np.float32, "image": np.uint8}
 QUERY = {"beta": 0, "cout": 1, "cin_g": 2, "groups": 3, "stride": 4, "n_groups": 5,
-         "n_patterns": 6, "image_bytes": 7, "fast_path": 8}
+         "n_patterns": 6, "image_bytes": 7, "fast_path": 8, "tensor_bytes": 9}
 _DT = {torch.float32: PP_F32, torch.float16: PP_F16}
 
 
@@ -43,6 +43,7 @@ class Layer:
     def __init__(self, handle: ctypes.c_void_p):
         self._h = handle
         self._dev_buf: Optional[torch.Tensor] = None
+        self._tensor_buf: Optional[torch.Tensor] = None
 
     # ---- host side
     def query(self, key: str) -> int:
@@ -84,7 +85,8 @@ class Layer:
 
     # ---- device side
     def bind(self, device=None, stream=None) -> "Layer":
-        """Copy the device image into a fresh torch buffer on ``device`` (async on ``stream``)."""
+        """Copy the device image into a fresh torch buffer on ``device`` and build the tensor-core
+        weights beside it where the layer has them (async on ``stream``)."""
         device = torch.device(device if device is not None else "cuda")
         if device.type != "cuda":
             raise ValueError("the packed image must live in CUDA device memory")
@@ -93,6 +95,13 @@ class Layer:
         _lib.check("pp_bind_device", _lib.load().pp_bind_device(
             self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
         self._dev_buf = buf
+        self._tensor_buf = None
+        n = self.query("tensor_bytes")
+        if n:
+            buf = torch.empty(n, dtype=torch.uint8, device=device)
+            _lib.check("pp_bind_tensor", _lib.load().pp_bind_tensor(
+                self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
+            self._tensor_buf = buf
         return self
 
     def out_shape(self, x_shape) -> tuple:
@@ -122,6 +131,20 @@ class Layer:
                  "chunks": int(info[3]), "rows_or_planes": int(info[4]), "stages": int(info[5]),
                  "warps": int(info[6]), "smem_bytes": int(info[10]), "ctas": int(info[12])}
         return d
+
+    TENSOR_PLAN_KEYS = ("tensor", "splits", "workspace_bytes", "units", "positions", "filters",
+                        "tile_w", "tile_h")
+
+    def tensor_plan(self, x_shape, workspace_bytes: int = 0, pool2x2: bool = False,
+                    dtype=torch.float32) -> dict:
+        """Whether a bound layer's call takes the tensor-core kernel (``tensor`` 1) and its plan
+        there (pp_conv_tensor_plan); ``plan`` describes the calls that do not."""
+        N, _, H, W = x_shape
+        n = len(self.TENSOR_PLAN_KEYS)
+        info = (ctypes.c_int64 * n)()
+        _lib.check("pp_conv_tensor_plan", _lib.load().pp_conv_tensor_plan(
+            self._h, _DT[dtype], 1 if pool2x2 else 0, N, H, W, int(workspace_bytes), info, n))
+        return dict(zip(self.TENSOR_PLAN_KEYS, (int(v) for v in info)))
 
     def workspace_bytes(self, x_shape, pool2x2: bool = False, dtype=torch.float32) -> int:
         """Workspace the call would use for this input shape and dtype (0: none): the input-channel

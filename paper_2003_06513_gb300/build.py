@@ -1,7 +1,7 @@
 """Build libpatconv.so in-tree: nvcc for the sm_103a kernels, g++ for the host packer.
 
 The library is written to ``paper_2003_06513_gb300/_build/libpatconv.so`` (git-ignored) and is
-rebuilt whenever a source file or a flag changes.  No CMake: two translation units compiled in
+rebuilt whenever a source file or a flag changes.  No CMake: three translation units compiled in
 parallel and one link, so a fresh build takes well under a minute.
 """
 from __future__ import annotations
@@ -24,7 +24,7 @@ NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "--expt-relaxed-constexpr", "-Xc
               "-Xcompiler", "-ffp-contract=off", "-I", os.path.join(ROOT, "include")] + ARCH
 GXX_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-ffp-contract=off", "-Wall", "-I",
              os.path.join(ROOT, "include")]
-SOURCES = ["conv.cu", "pack.cpp", "layer.h", "gen_dispatch.py"]
+SOURCES = ["conv.cu", "tensor.cu", "tensor.h", "pack.cpp", "layer.h", "gen_dispatch.py"]
 
 
 def _nvcc() -> str:
@@ -56,9 +56,11 @@ def build(force: bool = False, verbose: bool = False, extra_nvcc=()) -> str:
     subprocess.run([sys.executable, os.path.join(CSRC, "gen_dispatch.py"),
                     os.path.join(BUILD, "pattern_dispatch.h")], check=True)
     conv_o = os.path.join(BUILD, "conv.o")
+    tensor_o = os.path.join(BUILD, "tensor.o")
     pack_o = os.path.join(BUILD, "pack.o")
     cmds = [
         [nvcc, "-c", os.path.join(CSRC, "conv.cu"), "-o", conv_o, "-I", BUILD] + NVCC_FLAGS + list(extra_nvcc),
+        [nvcc, "-c", os.path.join(CSRC, "tensor.cu"), "-o", tensor_o] + NVCC_FLAGS + list(extra_nvcc),
         ["g++", "-c", os.path.join(CSRC, "pack.cpp"), "-o", pack_o] + GXX_FLAGS,
     ]
 
@@ -70,10 +72,10 @@ def build(force: bool = False, verbose: bool = False, extra_nvcc=()) -> str:
             raise RuntimeError(f"build step failed: {' '.join(cmd[:3])}")
         return r.stdout + r.stderr
 
-    with ThreadPoolExecutor(max_workers=2) as ex:
+    with ThreadPoolExecutor(max_workers=3) as ex:
         list(ex.map(run, cmds))
     tmp = LIB + ".tmp"
-    run([nvcc, "-shared", "-o", tmp, conv_o, pack_o] + ARCH + ["-cudart", "static"])
+    run([nvcc, "-shared", "-o", tmp, conv_o, tensor_o, pack_o] + ARCH + ["-cudart", "static"])
     os.replace(tmp, LIB)
     with open(stamp, "w") as f:
         f.write(digest)

@@ -52,6 +52,7 @@
 #include "../../include/patconv.h"
 #include "layer.h"
 #include "pattern_dispatch.h"
+#include "tensor.h"
 
 using namespace patconv;
 
@@ -2267,6 +2268,8 @@ struct Plan {
     int streamk = 0;              // balanced schedule over sm_count() CTAs (KS = 1)
     int dg = 1;                   // stride 2: filter groups per warp (2: 8 warps of 16 slots)
     size_t ws_bytes = 0;          // workspace the chosen split or schedule needs (0: none)
+    bool tensor = false;          // a layer bound for it takes the tensor-core kernel, as planned in tc
+    TensorPlan tc;
 };
 
 // Workspace of the balanced schedule over P CTAs: a slot of raw accumulators per CTA, then a flag
@@ -2644,6 +2647,20 @@ int make_plan_uncached(const pp_layer* L, int N, int H, int W, size_t ws_avail, 
 // (channel, group), 0.87 at 2.4 and 1 from 8 on.
 double shift_gain(double kept_per_channel) { return std::min(1.0, 0.82 + 0.0225 * kept_per_channel); }
 
+// Whether a call takes the tensor-core kernel: where its estimate is the lower one, and for fp32 only
+// where its rounding error is no larger.  The FFMA kernel's error grows with the number of products
+// it adds one after the other (1.1e-7 of the result at 77, 2.2e-7 at 307, 2.7e-7 at 614; 7e-8 at
+// 12), the tensor cores' starts at 0.9e-7 (the fp16 pairs) and grows slower (1.25e-7 at 307, 1.45e-7
+// at 614).
+bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int es) {
+    const double products = 4.0 * L->beta / L->cout;
+    if (es == 4 && products < 72.0 * pl.KS) return false;
+    if (!L->fast) return true;
+    const double flop = 8.0 * L->beta * (double)N * Ho * Wo;
+    const double rate = (es == 4 ? 28e6 : 24e6) * (L->stride == 2 ? 0.5 : 1.0);   // FLOP a microsecond
+    return pl.tc.clocks / 1900.0 + 3.0 < 0.95 * (flop / rate + 8.0);
+}
+
 int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out, int pool = 0,
               bool allow_sk = true, int es = 4) {
     pp_layer* ML = const_cast<pp_layer*>(L);   // the cache is the only mutable part of a handle
@@ -2674,6 +2691,8 @@ int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out
             cs * shift_gain(kpc) < cost)
             pl = ps;
     }
+    pl.tensor = tensor_plan(L, N, H, W, pool, es, ws_avail, sm_count(), &pl.tc) &&
+                tensor_wins(L, pl, N, (H - 1) / L->stride + 1, (W - 1) / L->stride + 1, es);
     std::lock_guard<std::mutex> g(cache->mu);
     if (cache->plans.size() >= 256) cache->plans.clear();
     cache->plans[key] = pl;
@@ -2851,6 +2870,67 @@ TmKernel pick_tm(bool sk, size_t smem, bool* ok, int dg = 1) {
     return nullptr;
 }
 
+// Reduction of an input-channel split: KS planes of partial sums to the output.
+template <typename T>
+int launch_reduce(const float* wsf, void* y, const float* bias, int ks, size_t total, int cout, int Ho, int Wo, int relu,
+                  int pool, cudaStream_t st) {
+    // threads: pooled outputs, or quads of outputs where the reduction loads 16 bytes a split
+    // and there are enough of them to give every SM 512 threads (smaller outputs take more
+    // threads, one element each: 64x64 32x32 N=1 16.1 us, in quads 16.8 us)
+    const int quads = total % 4 == 0 && reinterpret_cast<uintptr_t>(wsf) % 16 == 0 &&
+                      total / 4 >= (size_t)sm_count() * 512;
+    const size_t items = pool ? total / 4 : (quads ? total / 4 : total);
+    const unsigned blocks = (unsigned)std::max<size_t>(1, std::min<size_t>((items + 255) / 256, (size_t)sm_count() * 16));
+    T* yt = static_cast<T*>(y);
+    const int hw = Ho * Wo;
+    const cudaError_t e = pool ? launch(splitk_reduce_pool<T>, blocks, 256, 0, st, wsf, yt, bias, ks, total, cout, Ho, Wo, relu)
+                               : launch(splitk_reduce<T>, blocks, 256, 0, st, wsf, yt, bias, ks, total, cout, hw, relu, quads);
+    return e == cudaSuccess ? PP_OK : PP_ERR_CUDA;
+}
+
+// The tensor-core kernel can be switched off (PATCONV_TENSOR=0).
+bool tensor_enabled() {
+    static const bool on = [] {
+        const char* e = std::getenv("PATCONV_TENSOR");
+        return !(e && e[0] == '0');
+    }();
+    return on;
+}
+
+template <typename T>
+int launch_tensor(const pp_layer* L, const TensorPlan& pl, const void* x, void* y, const float* bias, int relu, int N,
+                  int H, int W, int Ho, int Wo, void* ws, cudaStream_t st, int pool) {
+    TensorCall c{};
+    c.L = L;
+    c.x = x;
+    c.y = y;
+    c.bias = bias;
+    c.relu = relu;
+    c.N = N;
+    c.H = H;
+    c.W = W;
+    c.Ho = Ho;
+    c.Wo = Wo;
+    c.pool = pool;
+    c.es = (int)sizeof(T);
+    c.ws = ws;
+    c.status = status_word();
+    if (!c.status) return PP_ERR_CUDA;
+    const bool inject = g_inject_timeout.exchange(0) != 0;
+    c.wait_limit = inject ? kInjectedWaitCycles : kTimeoutCycles;
+    c.no_fill = inject ? 1 : 0;
+    c.sms = sm_count();
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool captured = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    c.pdl = pdl_enabled() && !captured;
+    c.st = st;
+    if (tensor_launch(c, pl) != cudaSuccess) return PP_ERR_CUDA;
+    if (pl.KS > 1)
+        return launch_reduce<T>(static_cast<const float*>(ws), y, bias, pl.KS, (size_t)N * L->cout * Ho * Wo, L->cout, Ho,
+                                Wo, relu, pool, st);
+    return PP_OK;
+}
+
 template <int S, typename T>
 int launch_tm(const pp_layer* L, const void* x, void* y, const float* bias, int relu, int N, int H, int W, int Ho,
               int Wo, void* ws, size_t ws_bytes, cudaStream_t st, int pool = 0) {
@@ -2860,6 +2940,8 @@ int launch_tm(const pp_layer* L, const void* x, void* y, const float* bias, int 
     if ((pl.KS > 1 || pl.streamk) && reinterpret_cast<uintptr_t>(ws) % 16 != 0) return PP_ERR_ALIGN;
     // never planned: pool windows must lie in one block; blocks at 4j - 2 are fp32 only
     if ((pool && pl.shift == 1) || (pl.shift == 2 && sizeof(T) != 4)) return PP_ERR_SHAPE;
+    if (pl.tensor && L->tdev && tensor_enabled())
+        return launch_tensor<T>(L, pl.tc, x, y, bias, relu, N, H, W, Ho, Wo, ws, st, pool);
     TmParams p{};
     p.x = x;
     p.y = y;
@@ -2985,22 +3067,7 @@ int launch_tm(const pp_layer* L, const void* x, void* y, const float* bias, int 
                                                          (units + kMaxUnitsPerCta - 1) / kMaxUnitsPerCta)
                                    : units;
     if (launch(kern, (unsigned)ctas, kThreadsTM / pl.dg, smem, st, p, tmap) != cudaSuccess) return PP_ERR_CUDA;
-    if (pl.KS > 1) {
-        const size_t total = p.ws_stride;
-        const float* wsf = p.ws;
-        // threads: pooled outputs, or quads of outputs where the reduction loads 16 bytes a split
-        // and there are enough of them to give every SM 512 threads (smaller outputs take more
-        // threads, one element each: 64x64 32x32 N=1 16.1 us, in quads 16.8 us)
-        const int quads = total % 4 == 0 && reinterpret_cast<uintptr_t>(wsf) % 16 == 0 &&
-                          total / 4 >= (size_t)sm_count() * 512;
-        const size_t items = pool ? total / 4 : (quads ? total / 4 : total);
-        const unsigned blocks = (unsigned)std::max<size_t>(1, std::min<size_t>((items + 255) / 256, (size_t)sm_count() * 16));
-        T* yt = static_cast<T*>(y);
-        const int ks = pl.KS, cout = L->cout, hw = Ho * Wo;
-        const cudaError_t e = pool ? launch(splitk_reduce_pool<T>, blocks, 256, 0, st, wsf, yt, bias, ks, total, cout, Ho, Wo, relu)
-                                   : launch(splitk_reduce<T>, blocks, 256, 0, st, wsf, yt, bias, ks, total, cout, hw, relu, quads);
-        if (e != cudaSuccess) return PP_ERR_CUDA;
-    }
+    if (pl.KS > 1) return launch_reduce<T>(p.ws, y, bias, pl.KS, p.ws_stride, L->cout, Ho, Wo, relu, pool, st);
     return PP_OK;
 }
 
@@ -3361,6 +3428,11 @@ int launch_depthwise(const pp_layer* L, const void* x, void* y, const float* bia
 template <typename T>
 int launch_generic(const pp_layer* L, const void* x, void* y, const float* bias, int relu, int N, int H, int W,
                    int Ho, int Wo, cudaStream_t st) {
+    if (!L->depthwise && L->tdev && tensor_enabled()) {
+        Plan pl;
+        if (make_plan(L, N, H, W, 0, &pl, 0, true, (int)sizeof(T)) == PP_OK && pl.tensor)
+            return launch_tensor<T>(L, pl.tc, x, y, bias, relu, N, H, W, Ho, Wo, nullptr, st, 0);
+    }
     const unsigned char* img = static_cast<const unsigned char*>(L->dev);
     TapTable tt{};
     for (int p = 0; p < L->n_patterns; ++p) {
@@ -3413,6 +3485,19 @@ int pp_bind_device(pp_handle h, void* dev_image, size_t bytes, void* stream) {
         return PP_ERR_CUDA;
     h->dev = dev_image;
     h->dev_bytes = bytes;
+    h->tdev = nullptr;
+    return PP_OK;
+}
+
+int pp_bind_tensor(pp_handle h, void* dev, size_t bytes, void* stream) {
+    if (!h || !dev) return PP_ERR_NULL;
+    if (!h->dev) return PP_ERR_NOT_BOUND;
+    const size_t need = tensor_weight_bytes(h);
+    if (need == 0) return PP_ERR_PATH;
+    if (bytes < need) return PP_ERR_BUFFER;
+    if (reinterpret_cast<uintptr_t>(dev) % 256 != 0) return PP_ERR_ALIGN;
+    if (tensor_build_weights(h, dev, static_cast<cudaStream_t>(stream)) != cudaSuccess) return PP_ERR_CUDA;
+    h->tdev = dev;
     return PP_OK;
 }
 
@@ -3566,6 +3651,30 @@ int pp_conv_plan_dt(pp_handle h, int dtype, int pool, int N, int H, int W, size_
     if (pool != 0 && pool != 1) return PP_ERR_ARG;
     if (pool && h && (h->depthwise || !h->fast)) return PP_ERR_PATH;
     return conv_plan(h, N, H, W, workspace_bytes, info, n_info, pool, dtype == PP_F32 ? 4 : 2);
+}
+
+int pp_conv_tensor_plan(pp_handle h, int dtype, int pool, int N, int H, int W, size_t workspace_bytes, int64_t* info,
+                        int n_info) {
+    if (!h || !info) return PP_ERR_NULL;
+    if (dtype != PP_F32 && dtype != PP_F16) return PP_ERR_DTYPE;
+    if (pool != 0 && pool != 1) return PP_ERR_ARG;
+    if (pool && (h->depthwise || !h->fast)) return PP_ERR_PATH;
+    if (N < 1 || H < 1 || W < 1 || n_info < 1) return PP_ERR_SHAPE;
+    int64_t v[8] = {0};
+    Plan pl;
+    const size_t ws = h->fast ? workspace_bytes : 0;
+    if (!h->depthwise && make_plan(h, N, H, W, ws, &pl, pool, true, dtype == PP_F32 ? 4 : 2) == PP_OK && pl.tensor) {
+        v[0] = 1;
+        v[1] = pl.tc.KS;
+        v[2] = (int64_t)pl.tc.ws_bytes;
+        v[3] = pl.tc.units;
+        v[4] = 128 * pl.tc.MT;
+        v[5] = pl.tc.NC;
+        v[6] = pl.tc.tw;
+        v[7] = pl.tc.th;
+    }
+    for (int i = 0; i < n_info && i < 8; ++i) info[i] = v[i];
+    return PP_OK;
 }
 
 int pp_conv_workspace_size(pp_handle h, int N, int H, int W, size_t* bytes) {

@@ -50,6 +50,11 @@ struct pp_layer {
     void* dev = nullptr;               // caller-owned device copy of `image`
     size_t dev_bytes = 0;
 
+    // tensor-core weights (tensor.cu): fp16 pairs of the kept weights times 2^tc_exp
+    bool tc_ok = false;                // the pairs hold every kept weight (pack.cpp)
+    int tc_exp = 0;
+    void* tdev = nullptr;              // caller-owned device buffer, built by pp_bind_tensor
+
     // launch plans by call shape (conv.cu), created on the first plan by call_once, so that calls
     // from several host threads see it fully constructed
     std::unique_ptr<patconv::PlanCacheBase> plans;

@@ -18,6 +18,7 @@
 
 #include "../../include/patconv.h"
 #include "layer.h"
+#include "tensor.h"
 
 using namespace patconv;
 
@@ -153,6 +154,25 @@ int build(pp_layer* L, const float* W, double keep) {
         const int p = L->pid[k];
         if (p < 0) continue;
         for (int j = 0; j < 4; ++j) L->dense[9 * k + taps[p][j]] = W[9 * k + taps[p][j]];
+    }
+
+    // 6. may the tensor-core kernel hold the weights as fp16 pairs?  The pair of v 2^tc_exp, the
+    // layer's largest weight in [2^14, 2^15), has 22 bits down to 2^-28 of that weight and an
+    // absolute error of 2^-50 of it below; a filter whose own largest weight is 2^-20 of the
+    // layer's or less keeps the layer on the FFMA kernel, and so does a weight scale beyond
+    // 2^+-30 (the scales of weights and inputs are divided out in fp32).
+    L->tc_ok = false;
+    if (!L->depthwise) {
+        float top = 0.0f;
+        std::vector<float> fmax_(cout, 0.0f);
+        for (size_t k = 0; k < K; ++k)
+            for (int t = 0; t < 9; ++t) fmax_[k / cin_g] = std::max(fmax_[k / cin_g], std::fabs(L->dense[9 * k + t]));
+        for (int co = 0; co < cout; ++co) top = std::max(top, fmax_[co]);
+        const int e = top > 0.0f ? std::ilogb(top) : 99;
+        L->tc_ok = e >= -30 && e <= 30;
+        for (int co = 0; co < cout && L->tc_ok; ++co)
+            if (fmax_[co] > 0.0f && fmax_[co] < std::ldexp(top, -20)) L->tc_ok = false;
+        L->tc_exp = L->tc_ok ? 14 - e : 0;
     }
 
     const size_t b_perm = L->perm.size() * 4, b_desc = L->desc.size() * 8,
@@ -299,6 +319,7 @@ int pp_query(pp_handle h, int key, int64_t* value) {
         case PP_Q_N_PATTERNS: v = h->n_patterns; break;
         case PP_Q_IMAGE_BYTES: v = (int64_t)h->image.size(); break;
         case PP_Q_FAST_PATH: v = h->fast ? 1 : 0; break;
+        case PP_Q_TENSOR_BYTES: v = (int64_t)tensor_weight_bytes(h); break;
         default:
             if (key >= PP_Q_SECTION_BYTES && key <= PP_Q_SECTION_BYTES + PP_SEC_IMAGE) {
                 v = (int64_t)section_bytes(h, key - PP_Q_SECTION_BYTES);

@@ -1,0 +1,233 @@
+"""The tensor-core kernel against the float64 oracle, and the CUDA-core kernel beside it.
+
+Sizes sit where the kernel can go wrong: tiles of 128, 256 and 512 positions and their remainders,
+rectangles cut by the map's edge, odd maps, channel counts off the 16-channel blocks, filter counts
+off the multiples of 16 and over 256, odd numbers of tiles (the last CTA pair has half its work),
+both strides, both types, the fused pool, an input-channel split.  The bar is the other conv tests'
+(1e-4 of sum|W_hat||x| for fp32 I/O, 2e-3 for fp16); the fp32 cases also hold 4e-7 of the result in
+the 2-norm: the fp16 pairs carry 22 bits (2^-23 a factor), each chain truncates nine sums and up to
+32 of them are rounded once, 2e-7 in all, with a factor of two to spare."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import conv as OC
+from oracle import patterns as OP
+from oracle import project as OPR
+from paper_2003_06513_gb300 import _lib, api
+from paper_2003_06513_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"f32": 1e-4, "f16": 2e-3}
+NP = {"f32": np.float32, "f16": np.float16}
+
+
+@pytest.fixture(autouse=True)
+def _clean_status():
+    yield
+    torch.cuda.synchronize()
+    st = ctypes.c_uint(0)
+    assert _lib.load().pp_device_status(1, ctypes.byref(st)) == 0 and st.value == 0
+
+
+def _layer(cout, cin, keep, stride, seed, patterns=None):
+    rng = np.random.default_rng(seed)
+    W = (rng.standard_normal((cout, cin, 3, 3)) * np.sqrt(2 / (9 * cin))).astype(np.float32)
+    b = (rng.standard_normal(cout) * 0.1).astype(np.float32)
+    return api.pp_pack(W, patterns, keep, 1, stride).bind("cuda"), W, b
+
+
+def _cuda_cores_only(layer):
+    """Binding the device image again withdraws the tensor cores."""
+    buf = layer._dev_buf
+    _lib.check("pp_bind_device", _lib.load().pp_bind_device(
+        layer._h, ctypes.c_void_p(buf.data_ptr()), buf.numel(), None))
+    torch.cuda.synchronize()
+    return layer
+
+
+def _check(y, x, W, b, keep, stride, pool, io, masks=None, idx=None):
+    idx = list(range(x.shape[0])) if idx is None else idx
+    Wh = OPR.project(W, masks if masks is not None else OP.default8(), keep)["W_hat"]
+    xs = x[idx].astype(np.float64)
+    ref, den = OC.conv_ref(xs, Wh, b, stride, True), OC.denominator(xs, Wh, b, stride)
+    if pool:
+        ref, den = OC.maxpool2x2(ref), OC.maxpool2x2(den)
+    got = y[idx].double().cpu().numpy()
+    err = OC.max_norm_err(got, ref, den)
+    assert err <= TOL[io], f"max normalised error {err:.3e}"
+    if io == "f32":
+        rel = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+        assert rel <= 4e-7, f"relative error {rel:.3e}"
+
+
+CASES = [  # cout, cin, n, h, w, keep, io, stride, pool
+    (64, 64, 40, 32, 32, 0.5, "f32", 1, False),        # 512-position tiles
+    (64, 128, 17, 61, 59, 0.4, "f32", 1, False),       # odd map, odd batch
+    (96, 80, 9, 45, 61, 0.5, "f32", 1, False),         # 256-position tiles
+    (150, 90, 9, 45, 61, 0.5, "f32", 1, False),        # 160 filters of 150, 96 channels of 90
+    (40, 100, 60, 30, 30, 1.0, "f32", 1, False),       # 48 filters of 40
+    (300, 77, 16, 29, 31, 0.5, "f32", 1, False),       # two chunks of 160 filters, 300 of 320
+    (512, 144, 160, 7, 7, 0.5, "f32", 1, False),       # many images a tile
+    (256, 64, 3, 57, 211, 0.5, "f32", 1, False),       # wide rows
+    (128, 96, 24, 28, 28, 0.4, "f32", 2, False),       # stride 2, even map
+    (72, 96, 24, 29, 27, 0.5, "f32", 2, False),        # stride 2, odd map
+    (64, 64, 32, 56, 56, 0.5, "f32", 1, True),         # pool, 512-position rectangles
+    (128, 64, 16, 50, 46, 0.5, "f32", 1, True),        # pool, rectangles cut by the edge
+    (256, 72, 24, 29, 27, 0.5, "f32", 1, True),        # pool, odd map: last row and column dropped
+    (64, 64, 24, 56, 56, 0.5, "f32", 2, True),         # pool at stride 2
+    (256, 64, 16, 28, 28, 1.0, "f16", 1, False),
+    (90, 70, 16, 45, 37, 0.5, "f16", 1, False),
+    (128, 72, 24, 29, 27, 0.5, "f16", 2, False),
+    (200, 96, 24, 28, 28, 0.5, "f16", 1, True),
+]
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_tensor_kernel_matches_oracle(case):
+    cout, cin, n, h, w, keep, io, stride, pool = case
+    layer, W, b = _layer(cout, cin, keep, stride, cin + w)
+    x = WL.activations((n, cin, h, w), 7 + h, relu=True, dtype=NP[io])
+    xt = torch.from_numpy(x).cuda()
+    assert layer.tensor_plan(xt.shape, 0, pool, xt.dtype)["tensor"] == 1
+    shape = layer.out_shape(xt.shape)
+    if pool:
+        shape = shape[:2] + (shape[2] // 2, shape[3] // 2)
+    guard = torch.full((256 + int(np.prod(shape)) + 256,), float("nan"), dtype=xt.dtype, device="cuda")
+    y = guard[256:-256].view(shape)
+    layer.conv(xt, torch.from_numpy(b).cuda(), True, out=y, pool2x2=pool)
+    assert torch.isnan(guard[:256]).all() and torch.isnan(guard[-256:]).all()
+    _check(y, x, W, b, keep, stride, pool, io, idx=[0, n // 2, n - 1])
+
+
+def test_tensor_split_of_the_input_channels():
+    """Few tiles and a workspace: partial sums per channel range, added by the reduction."""
+    layer, W, b = _layer(256, 512, 1.0, 1, 3)
+    x = WL.activations((6, 512, 14, 14), 4, relu=True)
+    xt = torch.from_numpy(x).cuda()
+    ws = torch.full((1 << 22,), float("nan"), device="cuda")
+    plan = layer.tensor_plan(xt.shape, ws.numel() * 4)
+    if not plan["tensor"]:
+        pytest.skip("this shape takes the CUDA-core kernel")
+    y = layer.conv(xt, torch.from_numpy(b).cuda(), True, workspace=ws)
+    _check(y, x, W, b, 1.0, 1, False, "f32")
+
+
+def test_tensor_kernel_other_pattern_library():
+    masks = [0x01B, 0x036, 0x0D8, 0x1B0]                 # the four 2x2 corners
+    layer, W, b = _layer(128, 96, 0.5, 1, 8, masks)
+    x = WL.activations((4, 96, 28, 28), 5, relu=True)
+    xt = torch.from_numpy(x).cuda()
+    assert layer.tensor_plan(xt.shape)["tensor"] == 1
+    y = layer.conv(xt, torch.from_numpy(b).cuda(), True)
+    _check(y, x, W, b, 0.5, 1, False, "f32", masks=masks)
+
+
+def _sides(layer, W, x, stride, relu=False):
+    """Outputs of the tensor-core and the CUDA-core kernel and the weights, no bias."""
+    xt = torch.from_numpy(x).cuda()
+    assert layer.tensor_plan(xt.shape)["tensor"] == 1
+    a = layer.conv(xt, None, relu)
+    c = _cuda_cores_only(api.pp_pack(W, None, 0.5, 1, stride).bind("cuda")).conv(xt, None, relu)
+    return a.double().cpu().numpy(), c.double().cpu().numpy()
+
+
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("kind", ["1e20", "1e37", "1e-20", "halves", "channels", "images", "decay"])
+def test_values_of_any_scale(kind, stride):
+    """Scales the fp16 pairs cannot hold without a scale of their own, and mixtures no scale holds
+    (those units are summed in fp32): each output within 2e-6 of its own sum|w||x|."""
+    layer, W, _ = _layer(128, 96, 0.5, stride, 11)
+    rng = np.random.default_rng(2)
+    x = np.maximum(rng.standard_normal((12, 96, 40, 44)), 0)
+    if kind.startswith("1e"):
+        x = x * float(kind)
+    elif kind == "halves":
+        x[..., :22] *= 1e7
+        x[..., 22:] *= 1e-7
+    elif kind == "channels":
+        x[:, ::2] *= 1e8
+        x[:, 1::2] *= 1e-8
+    elif kind == "images":
+        x *= 10.0 ** rng.uniform(-15, 15, (12, 1, 1, 1))
+    else:
+        x = np.exp(-rng.uniform(0, 60, x.shape))
+    x = x.astype(np.float32)
+    got, _ = _sides(layer, W, x, stride)
+    Wh = OPR.project(W, OP.default8(), 0.5)["W_hat"]
+    idx = [0, 11]
+    xs = x[idx].astype(np.float64)
+    ref, den = OC.conv_ref(xs, Wh, None, stride, False), OC.denominator(xs, Wh, None, stride)
+    assert np.all(np.abs(got[idx] - ref) <= 2e-6 * den + 1e-44)
+
+
+@pytest.mark.parametrize("relu", [False, True])
+def test_infinities_and_nan_reach_the_outputs_of_kept_taps_only(relu):
+    layer, W, _ = _layer(128, 96, 0.5, 1, 12)
+    x = WL.activations((8, 96, 40, 44), 3, relu=True)
+    x[0, 5, 7, 9], x[3, 0, 0, 0], x[7, 95, 39, 43], x[2, 1, 20, 20] = np.inf, np.nan, -np.inf, 3e38
+    a, c = _sides(layer, W, x, 1, relu)
+    assert np.array_equal(np.isnan(a), np.isnan(c)) and np.array_equal(np.isinf(a), np.isinf(c))
+    f = np.isfinite(c)
+    assert np.allclose(a[f], c[f], rtol=1e-4, atol=1e-4 * np.abs(x[np.isfinite(x) & (x < 1e30)]).max())
+
+
+def test_inputs_at_any_element_alignment():
+    layer, W, b = _layer(64, 64, 0.5, 1, 13)
+    x = WL.activations((16, 64, 40, 40), 6, relu=True)
+    for dt, io in ((torch.float32, "f32"), (torch.float16, "f16")):
+        buf = torch.zeros(x.size + 3, dtype=dt, device="cuda")
+        xt = buf[3:].view(x.shape)
+        xt.copy_(torch.from_numpy(x))
+        y = layer.conv(xt, torch.from_numpy(b).cuda(), True)
+        _check(y, xt.cpu().numpy(), W, b, 0.5, 1, False, io, idx=[0, 15])
+
+
+def test_same_result_every_time():
+    layer, _, b = _layer(256, 128, 0.4, 1, 14)
+    xt = torch.from_numpy(WL.activations((16, 128, 28, 28), 6, relu=True)).cuda()
+    bt = torch.from_numpy(b).cuda()
+    first = layer.conv(xt, bt, True)
+    for _ in range(3):
+        assert torch.equal(layer.conv(xt, bt, True), first)
+
+
+@pytest.mark.parametrize("case", [  # the CUDA-core kernel's schedules, without the tensor cores
+    (256, 256, 8, 28, 0.3, "f32", False, 1), (512, 512, 32, 28, 0.3, "f32", True, 1),
+    (128, 128, 16, 56, 0.3, "f32", False, 1), (128, 128, 64, 28, 1.0, "f32", False, 1),
+    (512, 512, 32, 14, 0.3, "f32", False, 1), (128, 128, 16, 56, 0.4, "f32", False, 2),
+    (256, 256, 11, 56, 0.3, "f16", False, 1), (256, 128, 8, 28, 0.4, "f16", False, 2)])
+def test_cuda_core_kernel_without_tensor_binding(case):
+    cout, cin, n, h, keep, io, pool, stride = case
+    layer, W, b = _layer(cout, cin, keep, stride, 20 + h)
+    _cuda_cores_only(layer)
+    x = WL.activations((n, cin, h, h), 30 + h, relu=True, dtype=NP[io])
+    xt = torch.from_numpy(x).cuda()
+    nb = layer.workspace_bytes(xt.shape, pool, xt.dtype)
+    ws = torch.empty(max(nb // 4, 1), device="cuda") if nb else None
+    y = layer.conv(xt, torch.from_numpy(b).cuda(), True, workspace=ws, pool2x2=pool)
+    Wh = OPR.project(W, OP.default8(), keep)["W_hat"]
+    idx = [0, n - 1]
+    xs = x[idx].astype(np.float64)
+    ref, den = OC.conv_ref(xs, Wh, b, stride, True), OC.denominator(xs, Wh, b, stride)
+    if pool:
+        ref, den = OC.maxpool2x2(ref), OC.maxpool2x2(den)
+    assert OC.max_norm_err(y[idx].double().cpu().numpy(), ref, den) <= TOL[io]
+
+
+def test_bind_tensor_errors():
+    lib = _lib.load()
+    layer, W, _ = _layer(32, 32, 0.5, 1, 15)
+    n = layer.query("tensor_bytes")
+    buf = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+    p = lambda o=0: ctypes.c_void_p(buf.data_ptr() + o)
+    assert lib.pp_bind_tensor(None, p(), n, None) == -1
+    assert lib.pp_bind_tensor(layer._h, None, n, None) == -1
+    assert lib.pp_bind_tensor(layer._h, p(), n - 1, None) == -9
+    assert lib.pp_bind_tensor(layer._h, p(16), n, None) == -6
+    assert lib.pp_bind_tensor(api.pp_pack(W, None, 0.5)._h, p(), n, None) == -8
+    dw = api.pp_pack(W[:, :1], None, 1.0, 32).bind("cuda")
+    assert dw.query("tensor_bytes") == 0 and lib.pp_bind_tensor(dw._h, p(), n, None) == -14
