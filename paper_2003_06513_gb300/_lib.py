@@ -59,6 +59,8 @@ _lib = None
 def load(build_if_missing: bool = True) -> ctypes.CDLL:
     """Load (building first if needed) and return the library with typed signatures."""
     global _lib
+    if _lib is not None:     # set once, fully typed
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

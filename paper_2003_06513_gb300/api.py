@@ -37,11 +37,22 @@ def _stream_ptr(stream, device) -> ctypes.c_void_p:
     return ctypes.c_void_p(int(s.cuda_stream))
 
 
+def _raw_stream(stream, device) -> int:
+    """The stream's handle; the current stream without building a Stream object (1 us a call)."""
+    if stream is not None:
+        return int(stream.cuda_stream)
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(index if index is not None else torch.cuda.current_device())
+
+
 class Layer:
     """A packed pattern-pruned 3x3 layer (handle of pp_pack)."""
 
     def __init__(self, handle: ctypes.c_void_p):
         self._h = handle
+        # immutable scalars, read once: a query is a foreign call (0.7 us), and conv needs four
+        self._cout, self._cin_g = self.query("cout"), self.query("cin_g")
+        self._stride, self._depthwise = self.query("stride"), self.query("groups") != 1
         self._dev_buf: Optional[torch.Tensor] = None
         self._tensor_buf: Optional[torch.Tensor] = None
 
@@ -69,19 +80,19 @@ class Layer:
 
     @property
     def cout(self) -> int:
-        return self.query("cout")
+        return self._cout
 
     @property
     def cin_g(self) -> int:
-        return self.query("cin_g")
+        return self._cin_g
 
     @property
     def stride(self) -> int:
-        return self.query("stride")
+        return self._stride
 
     @property
     def depthwise(self) -> bool:
-        return self.query("groups") != 1
+        return self._depthwise
 
     # ---- device side
     def bind(self, device=None, stream=None) -> "Layer":
@@ -158,34 +169,38 @@ class Layer:
         the 2x2/2 max-pool of that map, fused into the conv (pp_conv_pool_ws)."""
         if self._dev_buf is None:
             self.bind(x.device)
-        if not x.is_cuda or x.dtype not in _DT or not x.is_contiguous() or x.dim() != 4:
+        dt = _DT.get(x.dtype)
+        if not x.is_cuda or dt is None or not x.is_contiguous() or x.dim() != 4:
             raise ValueError("x must be a contiguous 4-d CUDA float32/float16 tensor (NCHW)")
-        cin = self.cout if self.depthwise else self.cin_g
-        if x.shape[1] != cin:
-            raise ValueError(f"x has {x.shape[1]} channels, layer expects {cin}")
-        shape = self.out_shape(tuple(x.shape))
+        N, C, H, W = x.shape
+        cout, st = self._cout, self._stride
+        cin = cout if self._depthwise else self._cin_g
+        if C != cin:
+            raise ValueError(f"x has {C} channels, layer expects {cin}")
+        shape = (N, cout, (H - 1) // st + 1, (W - 1) // st + 1)
         if pool2x2:
             shape = shape[:2] + (shape[2] // 2, shape[3] // 2)
         if out is None:
             out = torch.empty(shape, dtype=x.dtype, device=x.device)
-        if tuple(out.shape) != shape or out.dtype != x.dtype or not out.is_contiguous() or not out.is_cuda:
+        elif out.shape != shape or out.dtype != x.dtype or not out.is_contiguous() or not out.is_cuda:
             raise ValueError(f"out must be a contiguous CUDA tensor of shape {shape} and x's dtype")
         bptr = None
         if bias is not None:
-            if not bias.is_cuda or bias.dtype != torch.float32 or bias.numel() != self.cout \
+            if not bias.is_cuda or bias.dtype != torch.float32 or bias.numel() != cout \
                     or not bias.is_contiguous():
                 raise ValueError("bias must be a contiguous CUDA float32 tensor of Cout values")
-            bptr = ctypes.c_void_p(bias.data_ptr())
-        N, _, H, W = x.shape
+            bptr = bias.data_ptr()
         wptr, wbytes = None, 0
         if workspace is not None:
             if not workspace.is_cuda or not workspace.is_contiguous():
                 raise ValueError("workspace must be a contiguous CUDA tensor")
-            wptr, wbytes = ctypes.c_void_p(workspace.data_ptr()), workspace.numel() * workspace.element_size()
-        name = "pp_conv_pool_ws" if pool2x2 else "pp_conv_ws"
-        _lib.check(name, getattr(_lib.load(), name)(
-            self._h, ctypes.c_void_p(x.data_ptr()), _DT[x.dtype], N, H, W, bptr, int(bool(relu)),
-            ctypes.c_void_p(out.data_ptr()), wptr, wbytes, _stream_ptr(stream, x.device)))
+            wptr, wbytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
+        lib = _lib.load()
+        fn = lib.pp_conv_pool_ws if pool2x2 else lib.pp_conv_ws
+        rc = fn(self._h, x.data_ptr(), dt, N, H, W, bptr, 1 if relu else 0, out.data_ptr(), wptr, wbytes,
+                _raw_stream(stream, x.device))
+        if rc != 0:
+            raise _lib.PatconvError("pp_conv_pool_ws" if pool2x2 else "pp_conv_ws", rc)
         return out
 
     def __del__(self):
