@@ -38,7 +38,6 @@ constexpr int kMaxWSlots = 12, kMaxXStages = 4;
 constexpr int kRing = 6;                // items a producer thread's copies run ahead, plus one
 constexpr int kHdr = 8;                 // stage headers in flight
 constexpr unsigned kHeadBytes = 1024 + 2 * 256 * 4;   // barriers, headers, two units' biases
-constexpr unsigned kPoolBytes = 16384;
 constexpr uint32_t kTmemColumns = 512;
 constexpr float kWeightBias = 8.0e-8f;
 constexpr long long kDrainCycles = 2000000000LL;   // about one second
@@ -786,41 +785,64 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 if (lane == 0) mbar_arrive_leader(tempty + 8 * b);
             }
             if (bar_or<2, kPromoteWarps * 32>(!ok)) break;
-            const int HoWo = p.Ho * p.Wo;
             if (slow) {
                 general_unit<S, T>(p, U, threadIdx.x, M);
             } else if (p.pool && p.KS == 1) {
-                // 2x2 max-pool: a few filters of every position at a time through shared memory, a
-                // warp a filter.  MT 1: each half of the warps pools its own 128 filters.
+                // 2x2 max-pool: a few filters of every position at a time through shared memory, each
+                // row of outputs at an even pitch (a pooled output is two 8-byte loads), a warp a
+                // filter, a lane up to MT pooled outputs whose offsets are the same for every filter.
+                // MT 1: each half of the warps pools its own 128 filters.
                 constexpr int TPH = MT == 4 ? 2 : 1;          // tiles of a warp
                 constexpr int NF = MT == 4 ? 8 : 16;          // filters a step
                 constexpr int NW = MT == 1 ? 4 : 8;           // warps sharing them
-                float* pb = reinterpret_cast<float*>(smem + p.pool_off) + (MT == 1 ? half * NF * M : 0);
-                const int Hq = p.Ho >> 1, Wq = p.Wo >> 1;
-                const int py0 = U.oy0 >> 1, px0 = U.ox0 >> 1;   // pool tiles are rectangles of even size
-                const int rows = U.n < p.N ? min(p.th >> 1, Hq - py0) : 0, cols = min(p.tw >> 1, Wq - px0);
-                T* y = static_cast<T*>(p.y);
+                const int pitch = (p.tw + 1) & ~1, plane = p.th * pitch;
+                float* pb = reinterpret_cast<float*>(smem + p.pool_off) + (MT == 1 ? half * NF * plane : 0);
+                const int Hq = p.Ho >> 1, Wq = p.Wo >> 1, HqWq = Hq * Wq;
+                int wr[TPH];                                  // where this lane's positions go
+#pragma unroll
+                for (int i = 0; i < TPH; ++i) {
+                    const int pl = pos + 128 * (MT == 4 ? 2 * half + i : (MT == 2 ? half : 0));
+                    const int r = (int)fdiv((uint32_t)pl, p.d_wp), c = pl - r * p.Wp;
+                    wr[i] = r < p.th && c < p.tw ? r * pitch + c : -1;
+                }
+                int rd[MT], yo[MT];                           // this lane's pooled outputs
+                const int py0 = U.oy0 >> 1, px0 = U.ox0 >> 1, cols = p.tw >> 1;
+#pragma unroll
+                for (int i = 0; i < MT; ++i) {
+                    const int o = lane + 32 * i, r = o / max(cols, 1), c = o - r * cols;
+                    const bool in = U.n < p.N && 2 * r < p.th && cols > 0 && py0 + r < Hq && px0 + c < Wq;
+                    rd[i] = in ? 2 * r * pitch + 2 * c : -1;
+                    yo[i] = r * Wq + c;
+                }
+                T* y = static_cast<T*>(p.y) + ((size_t)U.n * p.Cout + U.r0) * HqWq + (size_t)py0 * Wq + px0;
+                const int nf = min(p.NC, p.Cout - U.r0);
 #pragma unroll
                 for (int fb = 0; fb < 128 / TPH / NF; ++fb) {
                     const int f0 = (MT == 1 ? 128 * half : 0) + NF * fb;
                     bar_or<2, kPromoteWarps * 32>(false);
 #pragma unroll
                     for (int i = 0; i < TPH; ++i) {
-                        const int pl = pos + 128 * (MT == 4 ? 2 * half + i : (MT == 2 ? half : 0));
+                        if (wr[i] >= 0) {
 #pragma unroll
-                        for (int k = 0; k < NF; ++k) pb[k * M + pl] = acc[i * 64 + NF * fb + k];
+                            for (int k = 0; k < NF; ++k) pb[k * plane + wr[i]] = acc[i * 64 + NF * fb + k];
+                        }
                     }
                     bar_or<2, kPromoteWarps * 32>(false);
-                    for (int f = warp % NW; f < NF; f += NW) {
-                        const int co = U.r0 + f0 + f;
-                        if (f0 + f >= p.NC || co >= p.Cout) break;
-                        const float b = s_bias[f0 + f];
-                        T* yc = y + (((size_t)U.n * p.Cout + co) * Hq + py0) * Wq + px0;
-                        for (int r = 0; r < rows; ++r) {
-                            const float* s = pb + f * M + 2 * r * p.Wp;
-                            for (int c = lane; c < cols; c += 32) {
-                                const float m = fmaxf(fmaxf(s[2 * c], s[2 * c + 1]), fmaxf(s[p.Wp + 2 * c], s[p.Wp + 2 * c + 1]));
-                                yc[(size_t)r * Wq + c] = out_of<T>(relu_of(m + b, p.relu));
+#pragma unroll
+                    for (int k = 0; k < NF / NW; ++k) {
+                        const int f = warp % NW + NW * k;
+                        if (f0 + f < nf) {
+                            const float b = s_bias[f0 + f];
+                            T* yf = y + (size_t)(f0 + f) * HqWq;
+#pragma unroll
+                            for (int i = 0; i < MT; ++i) {
+                                if (rd[i] >= 0) {
+                                    const float* q = pb + f * plane + rd[i];
+                                    const float2 u = *reinterpret_cast<const float2*>(q);
+                                    const float2 v = *reinterpret_cast<const float2*>(q + pitch);
+                                    const float m = fmaxf(fmaxf(u.x, u.y), fmaxf(v.x, v.y));
+                                    yf[yo[i]] = out_of<T>(relu_of(m + b, p.relu));
+                                }
                             }
                         }
                     }
@@ -832,13 +854,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                     const int pl = pos + 128 * (MT == 4 ? 2 * half + i : (MT == 2 ? half : 0));
                     const int f0 = MT == 1 ? 128 * half : 0;
                     const Point o = point_of(p, U, pl);
-                    const int nf = o.in ? min(p.NC, p.Cout - U.r0) - f0 : 0;   // filters to store
+                    // filters to store: one predicate a store, no branch (a branch every four filters
+                    // kept their loads and stores from overlapping: fp16 28x28 72 -> 84 us)
+                    const int nf = o.in ? min(p.NC, p.Cout - U.r0) - f0 : 0, HoWo = p.Ho * p.Wo;
                     const size_t o0 = (((size_t)o.n * p.Cout + U.r0 + f0) * p.Ho + o.oy) * p.Wo + o.ox;
                     if (p.KS > 1) {
                         float* w = p.ws + (size_t)U.ks * p.ws_stride + o0;
 #pragma unroll
                         for (int j = 0; j < NJ; ++j) {
-                            if (j < nf) w[(size_t)j * HoWo] = acc[i * 64 + j];
+                            if (j < nf) *w = acc[i * 64 + j];
+                            w += HoWo;
                         }
                     } else {
                         T* w = static_cast<T*>(p.y) + o0;
@@ -1141,7 +1166,7 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             c.mstep = M;
             tiles = (c.Q + M - 1) / M;
             c.P = S == 1 ? M + 2 * c.Wp + 2 : M + c.Wp + 1;
-            if (c.P / c.Ip + 2LL > (1LL << 30) / ((long long)L->cin_g * H * W)) continue;
+            if (c.P / c.Ip + 2LL > (1LL << 30) / ((long long)std::max(L->cin_g, L->cout) * H * W)) continue;
         } else {
             c.tw = (Wo + k - 1) / k;
             if (k > 1) c.tw = (c.tw + 1) / 2 * 2;
@@ -1159,7 +1184,7 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             tiles = (long long)N * c.tiles_x * c.tiles_y;
             c.P = S == 1 ? (th + 2) * c.Wp + 2 : (th + 1) * c.Wp + 1;
             c.Ip = 2;   // unused
-            if ((long long)L->cin_g * H * W >= (1LL << 30)) continue;
+            if ((long long)std::max(L->cin_g, L->cout) * H * W >= (1LL << 30)) continue;
         }
         if (tiles >= INT_MAX / 4) continue;
         c.tiles = (int)((tiles + 1) / 2);
@@ -1167,7 +1192,9 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         const int rows = S == 1 ? M + 2 * c.Wp + 2 : M + c.Wp + 1;
         c.plane = (unsigned)align_up((size_t)std::max(rows, c.P) * 16, 128);
         c.x_stage = c.plane * 2 * HL * (S == 1 ? 1 : 4);
-        c.tab_off = kHeadBytes + (pool ? kPoolBytes : 0);
+        // pooling: 32, 16 or 8 filters of a tile's outputs at an even row pitch
+        const size_t pool_bytes = pool ? (size_t)32 / c.MT * c.th * ((c.tw + 1) & ~1) * 4 : 0;
+        c.tab_off = (unsigned)(kHeadBytes + align_up(pool_bytes, 16));
         c.ring_off = (unsigned)align_up(c.tab_off + 4 * (size_t)c.P, 128);
         c.x_off = c.ring_off + (es == 4 ? kRing * 8 * kProducers * 4 : 0);
         if (c.x_off >= kSmemMax) continue;
