@@ -35,7 +35,7 @@ constexpr int kProducerWarps = 6;       // warps 8-13: input staging
 constexpr int kLoaderWarp = 14, kMmaWarp = 15;
 constexpr int kProducers = kProducerWarps * 32;
 constexpr int kMaxWSlots = 12, kMaxXStages = 4;
-constexpr int kRing = 6;                // items a producer thread's copies run ahead, plus one
+constexpr int kRing = 6, kRingPair = 4; // items a producer thread's copies run ahead, plus one
 constexpr int kHdr = 8;                 // stage headers in flight
 constexpr unsigned kHeadBytes = 1024 + 2 * 256 * 4;   // barriers, headers, two units' biases
 constexpr uint32_t kTmemColumns = 512;
@@ -77,7 +77,8 @@ struct TcParams {
     int tw, th, tiles_x, tiles_y;   // rectangles of tw x th outputs (tw 0: flat tiles)
     long long Q;
     int tiles, n_fchunks, n_units;
-    FastDiv d_ip, d_wp, d_p;
+    int ppr, n_entries, items;  // pixel pairs of a staged row (0: single pixels); table entries; items of a block
+    FastDiv d_ip, d_wp, d_p, d_ppr;
     float* ws;
     size_t ws_stride;
     int xs, hs, ls;            // input stages, slots of the hi and lo weights
@@ -379,22 +380,120 @@ __device__ __forceinline__ bool input_of(const TcParams& p, uint32_t t, int k, u
     return in;
 }
 
-// fp32 inputs, six warps: a thread takes items (plane, 8 channels, position), copies its eight
-// values asynchronously to its own column of a ring in shared memory (neighbouring lanes neighbouring
-// positions: coalesced), and kRing - 1 items later splits them and stores 16 bytes of hi and of lo.
-// The copies run ahead over blocks and units.  What held this part was the latency of its loads, not
-// their number or the arithmetic: two items ahead in registers kept six warps at a tenth of their
-// issue rate (0.85 clocks a value; vgg 64 -> 64 at 224x224 650 us).
-template <int S>
-__device__ __forceinline__ void produce_f32(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
+// asynchronous copy of n = 0 or BYTES bytes, zero-filled to BYTES
+template <int BYTES>
+__device__ __forceinline__ void copy_async(uint32_t dst, const char* src, uint32_t n) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(n), "n"(BYTES) : "memory");
+}
+
+// The first position of a flat tile's window as row and column of the padded grid.
+__device__ __forceinline__ void window_start(const TcParams& p, const Unit& U, int* row, int* col) {
+    const long long q = U.q0 - p.Wp - 1 + 2 * p.Wp;   // never negative
+    const uint32_t r = fdiv((uint32_t)q, p.d_wp);
+    *row = (int)r - 2;
+    *col = (int)((uint32_t)q - r * (uint32_t)p.Wp);
+}
+// Stride 1, even rows: entry m of a unit's table of pixel pairs, two neighbouring inputs of one row at
+// an even column.  x: the element offset from image n0's channel 0 (kOut: zeros); y: the first one's
+// position plus one in bits 0-15, bits 30 and 31 whether the first and the second are staged.
+__device__ __forceinline__ uint2 pair_entry(const TcParams& p, const Unit& U, int m, int n0) {
+    const int r = (int)fdiv((uint32_t)m, p.d_ppr), j = m - r * p.ppr;
+    int n, y, x, p0;
+    bool w0, w1;
+    if (p.tw) {
+        n = U.n;
+        y = U.oy0 + r - 1;
+        x = U.ox0 - 2 + 2 * j;
+        const int c = 2 * j - 1;
+        p0 = r * p.Wp + c;
+        w0 = c >= 0 && c < p.Wp;
+        w1 = c + 1 < p.Wp;
+        if (r >= p.th + 2) {   // the last entry: the two positions after the last row
+            y = -1;
+            p0 = r * p.Wp;
+            w0 = w1 = true;
+        }
+    } else {
+        int row, col;
+        window_start(p, U, &row, &col);
+        row += r;
+        x = 2 * j;
+        p0 = r * p.Wp + x - col;
+        w0 = p0 >= 0 && p0 < p.P && x < p.Wp;
+        w1 = p0 + 1 >= 0 && p0 + 1 < p.P && x + 1 < p.Wp;
+        y = -1;
+        n = 0;
+        if (row >= 0) {
+            n = (int)fdiv((uint32_t)row * (uint32_t)p.Wp, p.d_ip);
+            y = row - n * (p.Ho + 1);
+        }
+    }
+    uint2 e;
+    e.x = kOut;
+    if (n < p.N && y >= 0 && y < p.H && x >= 0 && x < p.W)
+        e.x = ((uint32_t)(n - n0) * (uint32_t)p.C * p.H + (uint32_t)y) * p.W + (uint32_t)x;
+    e.y = (w0 || w1 ? (uint32_t)(p0 + 1) : 0u) | (w0 ? 1u << 30 : 0u) | (w1 ? 1u << 31 : 0u);
+    return e;
+}
+
+// Staging by six warps: a thread takes items of eight channels, copies the item's values
+// asynchronously to its own column of a ring in shared memory (neighbouring lanes neighbouring
+// addresses), and RING - 1 items later splits them and stores 16 bytes of hi and of lo a position.
+// The copies run ahead over blocks and units.  What held this part was first the latency of its loads
+// (two items ahead in registers: 0.85 clocks a value), then the number of copies, a warp's copy of 4
+// bytes a lane taking some 16 clocks: so with PAIR (rows of even length, inputs aligned to two values)
+// a copy brings two values, two neighbouring positions at stride 1, a position's even and odd column
+// at stride 2 (256 -> 256, 28x28 to 14x14, batch 64: 64 -> 51 us).  fp16 inputs are exact: their 16
+// bits go to the stage as they are; the copy has no 2-byte form, so they come in pairs only.
+template <int S, typename T, bool PAIR>
+__device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
                                             volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
-    constexpr int NPL = S == 1 ? 1 : 4;
+    constexpr bool F32 = sizeof(T) == 4;
+    static_assert(F32 || PAIR, "fp16 values are copied in pairs");
+    constexpr int HL = F32 ? 2 : 1;
+    constexpr int V = PAIR ? 2 : 1;                  // values of a channel in an item
+    constexpr int WV = F32 ? V : 1;                  // words they take
+    constexpr int RING = WV == 2 ? kRingPair : kRing;
+    constexpr int SLOT = (8 * WV + 1) * kProducers;  // words of a ring slot: the values, where they go
     const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
-    const uint32_t HW = (uint32_t)p.H * p.W, HWB = HW * 4u;
+    const uint32_t HW = (uint32_t)p.H * p.W, HWB = HW * (uint32_t)sizeof(T);
     uint32_t* table = reinterpret_cast<uint32_t*>(smem + p.tab_off);
-    const int items = 2 * NPL * p.P, steps = (items + kProducers - 1) / kProducers;
-    const float* ring = reinterpret_cast<const float*>(smem + p.ring_off) + tid;
-    const uint32_t ring0 = smem_u32(ring);
+    uint2* table2 = reinterpret_cast<uint2*>(table);
+    const int steps = (p.items + kProducers - 1) / kProducers;
+    float* ring = reinterpret_cast<float*>(smem + p.ring_off);
+    const uint32_t second = S == 1 ? 16u : 2u * HL * p.plane;   // an item's second value: next position, or odd columns' plane
+    // item i of a unit, from a table entry: whether its inputs exist, their offset, and where it goes
+    // (byte offset in the stage; bits 30 and 31: the first and second value are staged)
+    auto decode = [&](int i, auto&& entry, uint32_t* off, uint32_t* dst) {
+        if (i >= p.items) {
+            *dst = 0;
+            return false;
+        }
+        if constexpr (S == 1 && PAIR) {
+            const int k = i >= p.n_entries ? 1 : 0;
+            const uint2 e = entry(i - k * p.n_entries);
+            *off = e.x + (k ? 8u * HW : 0u);
+            const uint32_t p1 = e.y & 0xFFFFu;   // position + 1
+            *dst = (e.y & 0xC0000000u) | (p1 * 16u + (uint32_t)k * p.plane);
+            return e.x != kOut;
+        } else {
+            const int k = (int)fdiv((uint32_t)i, p.d_p);
+            const int pos = i - k * p.P;
+            const uint32_t t = entry(pos).x;
+            bool in = t != kOut;
+            *off = (t >> 2) + ((k & 1) ? 8u * HW : 0u);
+            // planes at stride 2: 2 (odd rows) + (odd columns)
+            const int odd_row = PAIR ? k >> 1 : k >> 2, odd_col = PAIR ? 0 : (k >> 1) & 1;
+            if constexpr (S == 2) {
+                in = in && (!odd_col || (t & 1u)) && (!odd_row || (t & 2u));
+                *off += (uint32_t)odd_row * p.W + (uint32_t)odd_col;
+            }
+            const int pl = S == 1 ? 0 : 2 * odd_row + odd_col;
+            *dst = (PAIR ? 0xC0000000u : 0x40000000u) | ((uint32_t)(pl * 2 * HL + (k & 1)) * p.plane + (uint32_t)(pos + 1) * 16u);
+            return in;
+        }
+    };
+    auto channel_of = [&](int i) { return S == 1 && PAIR ? (i >= p.n_entries ? 8 : 0) : (int)(fdiv((uint32_t)i, p.d_p) & 1u) * 8; };
     int kexp = 0;
     Stage sg;
     // the copies' cursor: unit, block, step, slot
@@ -406,30 +505,36 @@ __device__ __forceinline__ void produce_f32(const TcParams& p, unsigned char* sm
                 const Unit U = unit_of(p, iu, rank);
                 const int n0 = first_image(p, U);
                 bar_or<1, kProducers>(false);
-                for (int i = tid; i < p.P; i += kProducers) table[i] = window_entry<S>(p, U, i, n0);
+                for (int i = tid; i < p.n_entries; i += kProducers) {
+                    if constexpr (S == 1 && PAIR) table2[i] = pair_entry(p, U, i, n0);
+                    else table[i] = window_entry<S>(p, U, i, n0);
+                }
                 bar_or<1, kProducers>(false);
                 icb = U.cb0;
                 icb1 = U.cb1;
                 ix = reinterpret_cast<const char*>(p.x) + ((size_t)n0 * p.C + U.cb0 * 16) * HWB;
             }
-            int k, pos;
-            uint32_t t = kOut, off;
-            if (item_of<S>(p, tid + ig * kProducers, items, &k, &pos)) {
-                t = table[pos];
-                const bool in = input_of<S>(p, t, k, HW, &off);
-                const int nch = in ? p.C - icb * 16 - 8 * (k & 1) : 0;
-                const char* src = in ? ix + (size_t)off * 4 : reinterpret_cast<const char*>(p.x);
-                const uint32_t dst = ring0 + (uint32_t)islot * (8 * kProducers * 4);
+            const int i = tid + ig * kProducers;
+            uint32_t off, dst;
+            const bool in = decode(i, [&](int m) {
+                if constexpr (S == 1 && PAIR) return table2[m];
+                else return make_uint2(table[m], 0u);
+            }, &off, &dst);
+            float* slot = ring + islot * SLOT;
+            reinterpret_cast<uint32_t*>(slot)[8 * WV * kProducers + tid] = dst;
+            if (dst != 0) {
+                const int nch = in ? p.C - icb * 16 - channel_of(i) : 0;
+                const char* src = in ? ix + (size_t)off * sizeof(T) : reinterpret_cast<const char*>(p.x);
+                const uint32_t to = smem_u32(slot + WV * tid);
                 if (nch >= 8 || nch <= 0) {
-                    const uint32_t n = nch > 0 ? 4u : 0u;
+                    const uint32_t n = nch > 0 ? 4u * WV : 0u;
                     const size_t step = nch > 0 ? HWB : 0;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j, src += step)
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + j * (kProducers * 4)), "l"(src), "r"(n) : "memory");
+                    for (int j = 0; j < 8; ++j, src += step) copy_async<4 * WV>(to + j * (4 * WV * kProducers), src, n);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + j * (kProducers * 4)), "l"(src), "r"(j < nch ? 4u : 0u) : "memory");
+                        copy_async<4 * WV>(to + j * (4 * WV * kProducers), src, j < nch ? 4u * WV : 0u);
                         if (j + 1 < nch) src += HWB;
                     }
                 }
@@ -439,90 +544,121 @@ __device__ __forceinline__ void produce_f32(const TcParams& p, unsigned char* sm
                 ix += (size_t)16 * HWB;
                 if (++icb == icb1) iu += pairs;
             }
-            if (++islot == kRing) islot = 0;
+            if (++islot == RING) islot = 0;
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int r = 0; r < kRing - 1; ++r) issue();
+    for (int r = 0; r < RING - 1; ++r) issue();
 
     int slot = 0;
     for (int u = pair; u < p.n_units; u += pairs) {
         const Unit U = unit_of(p, u, rank);
         for (int cb = U.cb0; cb < U.cb1; ++cb) {
             const bool ok = sg.e < p.xs || wait_bar(xempty + 8 * sg.s, (sg.ph & 1) ^ 1, p, abort_flag, kErrSpace);
-            unsigned char* st = smem + p.x_off + (size_t)sg.s * p.x_stage;
-            uint32_t mn = 0xFFFFFFFFu;
+            unsigned char* st = smem + p.x_off + (size_t)sg.s * p.x_stage - 16;   // positions are one too high
+            uint32_t mn = 0xFFFFFFFFu, bad = 0;
             __half2 hmx = __half2half2(__ushort_as_half(0));
             float scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
-            auto split = [&](const float (&v)[8], int i) {
-                int k, pos;
-                if (!item_of<S>(p, i, items, &k, &pos)) return;
-                // the smallest |v| as an ordered integer, a zero as the largest
+            auto split = [&](const float (&v)[WV][8], uint32_t dst) {
 #pragma unroll
-                for (int j = 0; j < 8; j += 2)
-                    mn = min(min(mn, 2u * __float_as_uint(v[j]) - 1u), 2u * __float_as_uint(v[j + 1]) - 1u);
-                uint4 hi, lo;
-                split8(v, scale, &hi, &lo, &hmx);
-                unsigned char* d = st + (uint32_t)((k >> 1) * 4 + (k & 1)) * p.plane + (uint32_t)pos * 16u;
-                *reinterpret_cast<uint4*>(d) = hi;
-                *reinterpret_cast<uint4*>(d + 2 * p.plane) = lo;
-            };
-            for (int g = 0; g < steps; ++g) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
-                float v[8];
+                for (int a = 0; a < V; ++a) {
+                    if (!(dst & (0x40000000u << a))) continue;
+                    unsigned char* d = st + (dst & 0x3FFFFFFFu) + a * second;
+                    if constexpr (!F32) {   // a word holds a channel's two values
+                        uint32_t w[4];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = ring[(slot * 8 + j) * kProducers];
-                issue();
-                if (++slot == kRing) slot = 0;
-                if (ok) split(v, tid + g * kProducers);
-            }
-            // the larger half of the largest hi parts; NaN is the largest of all
-            const uint32_t b = *reinterpret_cast<const uint32_t*>(&hmx);
-            uint32_t mx = max(b & 0xFFFFu, b >> 16);
-            if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
-            // hi parts up to 2^11 ... 2^15 use the pair's whole range; else the block is taken again
-            // (from memory), its largest value scaled to [2^13, 2^14)
-            int ex = (int)(mx >> 10) - 15 - kexp;
-            bool slow = false;
-            if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
-                const int n0 = first_image(p, U);
-                auto again = [&](int i, float (&v)[8]) {
-                    int k, pos;
-                    uint32_t off;
-                    const bool mine = item_of<S>(p, i, items, &k, &pos);
-                    const bool in = mine && input_of<S>(p, window_entry<S>(p, U, pos, n0), k, HW, &off);
-                    const float* src = static_cast<const float*>(p.x) + ((size_t)n0 * p.C + cb * 16) * HW + off;
-                    for (int j = 0; j < 8; ++j) v[j] = in && cb * 16 + 8 * (k & 1) + j < p.C ? __ldg(src + (size_t)j * HW) : 0.0f;
-                };
-                mx = 0;
-                float v[8];
-#pragma unroll 1
-                for (int g = 0; g < steps; ++g) {
-                    again(tid + g * kProducers, v);
+                        for (int j = 0; j < 4; ++j) {
+                            w[j] = __byte_perm(__float_as_uint(v[0][2 * j]), __float_as_uint(v[0][2 * j + 1]), a ? 0x7632 : 0x5410);
+                            bad |= ((w[j] & 0x7C007C00u) + 0x04000400u) & 0x80008000u;   // exponent 31: not finite
+                        }
+                        *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+                    } else {
+                        // the smallest |v| as an ordered integer, a zero as the largest
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[j]));
-                }
-                if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
-                ex = (int)(mx >> 24) - 127;
-                slow = ex < -60 || ex > 120;   // also infinities and NaN
-                if (!slow) {
-                    kexp = 13 - ex;
-                    scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
-#pragma unroll 1
-                    for (int g = 0; g < steps; ++g) {
-                        again(tid + g * kProducers, v);
-                        split(v, tid + g * kProducers);
+                        for (int j = 0; j < 8; j += 2)
+                            mn = min(min(mn, 2u * __float_as_uint(v[a][j]) - 1u), 2u * __float_as_uint(v[a][j + 1]) - 1u);
+                        uint4 hi, lo;
+                        split8(v[a], scale, &hi, &lo, &hmx);
+                        *reinterpret_cast<uint4*>(d) = hi;
+                        *reinterpret_cast<uint4*>(d + 2 * p.plane) = lo;
                     }
                 }
+            };
+            for (int g = 0; g < steps; ++g) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(RING - 2) : "memory");
+                float v[WV][8];
+                const float* from = ring + slot * SLOT;
+                const uint32_t dst = reinterpret_cast<const uint32_t*>(from)[8 * WV * kProducers + tid];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if constexpr (WV == 2) {
+                        const float2 t = *reinterpret_cast<const float2*>(from + 2 * (j * kProducers + tid));
+                        v[0][j] = t.x;
+                        v[WV - 1][j] = t.y;
+                    } else {
+                        v[0][j] = from[j * kProducers + tid];
+                    }
+                }
+                issue();
+                if (++slot == RING) slot = 0;
+                if (ok) split(v, dst);
             }
-            slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
+            bool slow = false;
+            if constexpr (!F32) {
+                if (!combine<false>(&bad, &mn, ok, red, &sg.par, warp, lane)) return;
+                slow = bad != 0;
+            } else {
+                // the larger half of the largest hi parts; NaN is the largest of all
+                const uint32_t b = *reinterpret_cast<const uint32_t*>(&hmx);
+                uint32_t mx = max(b & 0xFFFFu, b >> 16);
+                if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
+                // hi parts up to 2^11 ... 2^15 use the pair's whole range; else the block is taken again
+                // (from memory), its largest value scaled to [2^13, 2^14)
+                int ex = (int)(mx >> 10) - 15 - kexp;
+                if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
+                    const int n0 = first_image(p, U);
+                    auto again = [&](int i, float (&v)[V][8]) {
+                        uint32_t off, dst;
+                        const bool in = decode(i, [&](int m) {
+                            if constexpr (S == 1 && PAIR) return pair_entry(p, U, m, n0);
+                            else return make_uint2(window_entry<S>(p, U, m, n0), 0u);
+                        }, &off, &dst);
+                        const int nch = in ? p.C - cb * 16 - channel_of(i) : 0;
+                        const float* src = static_cast<const float*>(p.x) + ((size_t)n0 * p.C + cb * 16) * HW + off;
+                        for (int j = 0; j < 8; ++j)
+                            for (int a = 0; a < V; ++a) v[a][j] = j < nch ? __ldg(src + (size_t)j * HW + a) : 0.0f;
+                        return dst;
+                    };
+                    mx = 0;
+                    float v[V][8];
+    #pragma unroll 1
+                    for (int g = 0; g < steps; ++g) {
+                        const uint32_t dst = again(tid + g * kProducers, v);
+                        for (int a = 0; a < V; ++a)
+                            if (dst & (0x40000000u << a))
+                                for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[a][j]));
+                    }
+                    if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
+                    ex = (int)(mx >> 24) - 127;
+                    slow = ex < -60 || ex > 120;   // also infinities and NaN
+                    if (!slow) {
+                        kexp = 13 - ex;
+                        scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
+    #pragma unroll 1
+                        for (int g = 0; g < steps; ++g) {
+                            const uint32_t dst = again(tid + g * kProducers, v);
+                            split(v, dst);
+                        }
+                    }
+                }
+                slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
+            }
             publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
         }
     }
 }
 
-// fp16 inputs: exact, so the 16 bits go to the stage as they are.  Loads run two items ahead in
-// registers (the asynchronous copy has no 2-byte form).
+// fp16 rows of odd length, or inputs aligned to one value only: loads run two items ahead in registers.
 template <int S>
 __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
                                             volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
@@ -886,10 +1022,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
-            if constexpr (HL == 2) {
-                produce_f32<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
-                asm volatile("cp.async.wait_all;" ::: "memory");   // after a timeout: nothing in flight at the exit
-            } else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            if (p.ppr) produce_async<S, T, true>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            else if constexpr (HL == 2) produce_async<S, T, false>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            asm volatile("cp.async.wait_all;" ::: "memory");   // after a timeout: nothing in flight at the exit
         } else if (warp == kLoaderWarp) {
             // ---- weights: a slot holds this CTA's half of the unit's filters for a row of three
             // taps of a 16-channel block, [tap][8 channels][filter], the lo and hi parts in rings of
@@ -1195,8 +1331,25 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         // pooling: 32, 16 or 8 filters of a tile's outputs at an even row pitch
         const size_t pool_bytes = pool ? (size_t)32 / c.MT * c.th * ((c.tw + 1) & ~1) * 4 : 0;
         c.tab_off = (unsigned)(kHeadBytes + align_up(pool_bytes, 16));
-        c.ring_off = (unsigned)align_up(c.tab_off + 4 * (size_t)c.P, 128);
-        c.x_off = c.ring_off + (es == 4 ? kRing * 8 * kProducers * 4 : 0);
+        // items of a block: pairs of pixels where rows are even (and x is aligned to a pair:
+        // tensor_launch) unless that takes more rounds of the staging threads (fp16: as many); ppr is
+        // the pairs of a staged row, 0 with single pixels
+        const auto rounds_of = [](int n) { return (n + kProducers - 1) / kProducers; };
+        c.n_entries = c.P;
+        c.items = 2 * c.P * (S == 1 ? 1 : 4);
+        if (W % 2 == 0) {
+            const int ppr = S == 2 ? 2 : (c.tw ? (c.Wp + 2) / 2 : W / 2 + 1);
+            const int entries = S == 2 ? c.P : (c.tw ? (c.th + 2) * ppr + 1 : ((c.P + c.Wp - 1) / c.Wp + 1) * ppr);
+            const int items = S == 2 ? 4 * c.P : 2 * entries;
+            if (rounds_of(items) < rounds_of(c.items) + (es == 4 ? 1 : 0)) {
+                c.ppr = ppr;
+                c.n_entries = entries;
+                c.items = items;
+            }
+        }
+        if (c.P >= 0xFFFF) continue;
+        c.ring_off = (unsigned)align_up(c.tab_off + std::max<size_t>(4 * (size_t)c.P, 8 * (size_t)c.n_entries), 128);
+        c.x_off = c.ring_off + (es == 4 ? std::max(kRing * 9, kRingPair * 17) : kRing * 9) * kProducers * 4;
         if (c.x_off >= kSmemMax) continue;
         const size_t left = kSmemMax - c.x_off;
         // three input stages with two blocks' weights, else two with at least a block's and a row
@@ -1214,9 +1367,15 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         c.l_off = c.h_off + c.hs * c.w_slot;
         c.smem = c.l_off + (size_t)c.ls * c.w_slot;
         const long long units1 = (long long)c.tiles * c.n_fchunks, pairs = sms / 2;
-        // clocks of a 16-channel block (its MMAs, or its staging) and of a unit's stores
+        // clocks of a 16-channel block: its MMAs, and the rounds of staging that do not hide behind
+        // them (fitted to 19 layers with every tile each can take: within 10 %); rows of few outputs
+        // cost partial sectors, as 2.5 / width of the whole
         const double mma = 9.0 * (HL + 1) * c.MT * std::max(c.NC / 2.0, 32.0 + c.NC / 8.0) + 200.0;
-        const double stage = std::max(mma, 0.45 * 16.0 * c.P * (S == 1 ? 1 : 4));
+        const int rounds = rounds_of(c.items);
+        const double stage = es == 2 ? mma + 700.0 * std::max(0.0, rounds - (S == 1 ? 1.0 : 0.0))
+                             : c.ppr ? mma + 1000.0 * std::max(0.0, rounds - mma / 1900.0)
+                                     : mma + 600.0 * std::max(0.0, rounds - mma / 1000.0);
+        const double narrow = 1.0 + 2.5 / (c.tw ? c.tw : Wo);
         for (int ks = 1; ks <= c.n_cb; ++ks) {
             const int cbs = (c.n_cb + ks - 1) / ks;
             if ((c.n_cb + cbs - 1) / cbs != ks) continue;
@@ -1224,7 +1383,7 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             if (units1 * ks > INT_MAX / 2) break;
             const long long waves = (units1 * ks + pairs - 1) / pairs;
             const double stores = 128.0 * c.MT * c.NC * (ks > 1 ? 4 : es) / 10.0;
-            double t = waves * (std::max(cbs * stage, stores) + 1500.0) + 6000.0;
+            double t = waves * (std::max(cbs * stage, stores) + 1500.0) * narrow + 6000.0;
             if (ks > 1) t += 4000.0 + (double)ks * out_bytes / 2000.0;
             if (!have || t < best) {
                 have = true;
@@ -1265,6 +1424,9 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.Ip = pl.Ip;
     p.mstep = pl.mstep;
     p.P = pl.P;
+    p.ppr = pl.ppr;
+    p.n_entries = pl.n_entries;
+    p.items = pl.items;
     p.tw = pl.tw;
     p.th = pl.th;
     p.tiles_x = pl.tiles_x;
@@ -1276,6 +1438,7 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.d_ip = fast_div((uint32_t)pl.Ip);
     p.d_wp = fast_div((uint32_t)pl.Wp);
     p.d_p = fast_div((uint32_t)p.P);
+    p.d_ppr = fast_div((uint32_t)std::max(2, pl.ppr));
     p.ws = static_cast<float*>(c.ws);
     p.ws_stride = (size_t)c.N * L->cout * c.Ho * c.Wo;
     p.xs = pl.xs;
@@ -1290,6 +1453,11 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.x_off = pl.x_off;
     p.h_off = pl.h_off;
     p.l_off = pl.l_off;
+    if (pl.ppr && reinterpret_cast<uintptr_t>(c.x) % (2 * (size_t)c.es) != 0) {   // single pixels after all
+        p.ppr = 0;
+        p.n_entries = pl.P;
+        p.items = 2 * pl.P * (L->stride == 1 ? 1 : 4);
+    }
     TcKernel k;
     if (L->stride == 1) k = c.es == 4 ? pick<1, float>(pl.MT, pl.smem) : pick<1, __half>(pl.MT, pl.smem);
     else k = c.es == 4 ? pick<2, float>(pl.MT, pl.smem) : pick<2, __half>(pl.MT, pl.smem);

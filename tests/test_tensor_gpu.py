@@ -73,15 +73,15 @@ CASES = [  # cout, cin, n, h, w, keep, io, stride, pool
     (300, 77, 16, 29, 31, 0.5, "f32", 1, False),       # two chunks of 160 filters, 300 of 320
     (512, 144, 160, 7, 7, 0.5, "f32", 1, False),       # many images a tile
     (256, 64, 3, 57, 211, 0.5, "f32", 1, False),       # wide rows
-    (128, 96, 24, 28, 28, 0.4, "f32", 2, False),       # stride 2, even map
-    (72, 96, 24, 29, 27, 0.5, "f32", 2, False),        # stride 2, odd map
+    (128, 96, 64, 28, 28, 0.4, "f32", 2, False),       # stride 2, even map
+    (72, 96, 64, 29, 27, 0.5, "f32", 2, False),        # stride 2, odd map
     (64, 64, 32, 56, 56, 0.5, "f32", 1, True),         # pool, 512-position rectangles
     (128, 64, 16, 50, 46, 0.5, "f32", 1, True),        # pool, rectangles cut by the edge
     (256, 72, 24, 29, 27, 0.5, "f32", 1, True),        # pool, odd map: last row and column dropped
-    (64, 64, 24, 56, 56, 0.5, "f32", 2, True),         # pool at stride 2
+    (64, 64, 64, 56, 56, 0.5, "f32", 2, True),         # pool at stride 2
     (256, 64, 16, 28, 28, 1.0, "f16", 1, False),
     (90, 70, 16, 45, 37, 0.5, "f16", 1, False),
-    (128, 72, 24, 29, 27, 0.5, "f16", 2, False),
+    (128, 72, 64, 29, 27, 0.5, "f16", 2, False),
     (200, 96, 24, 28, 28, 0.5, "f16", 1, True),
 ]
 
