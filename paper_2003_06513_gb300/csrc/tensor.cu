@@ -35,7 +35,8 @@ constexpr int kProducerWarps = 6;       // warps 8-13: input staging
 constexpr int kLoaderWarp = 14, kMmaWarp = 15;
 constexpr int kProducers = kProducerWarps * 32;
 constexpr int kMaxWSlots = 12, kMaxXStages = 4;
-constexpr int kRing = 6, kRingPair = 4; // items a producer thread's copies run ahead, plus one
+// items a producer thread's copies run ahead, plus one, by the words of a channel in an item
+constexpr int ring_of(int words) { return words == 1 ? 6 : (words == 2 ? 4 : 3); }
 constexpr int kHdr = 8;                 // stage headers in flight
 constexpr unsigned kHeadBytes = 1024 + 2 * 256 * 4;   // barriers, headers, two units' biases
 constexpr uint32_t kTmemColumns = 512;
@@ -77,7 +78,7 @@ struct TcParams {
     int tw, th, tiles_x, tiles_y;   // rectangles of tw x th outputs (tw 0: flat tiles)
     long long Q;
     int tiles, n_fchunks, n_units;
-    int ppr, n_entries, items;  // pixel pairs of a staged row (0: single pixels); table entries; items of a block
+    int vec, ppr, n_entries, items;   // values a copy; copies of a staged row (vec > 1); table entries; items of a block
     FastDiv d_ip, d_wp, d_p, d_ppr;
     float* ws;
     size_t ws_stride;
@@ -383,7 +384,10 @@ __device__ __forceinline__ bool input_of(const TcParams& p, uint32_t t, int k, u
 // asynchronous copy of n = 0 or BYTES bytes, zero-filled to BYTES
 template <int BYTES>
 __device__ __forceinline__ void copy_async(uint32_t dst, const char* src, uint32_t n) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(n), "n"(BYTES) : "memory");
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(n), "n"(BYTES) : "memory");
 }
 
 // The first position of a flat tile's window as row and column of the padded grid.
@@ -393,34 +397,36 @@ __device__ __forceinline__ void window_start(const TcParams& p, const Unit& U, i
     *row = (int)r - 2;
     *col = (int)((uint32_t)q - r * (uint32_t)p.Wp);
 }
-// Stride 1, even rows: entry m of a unit's table of pixel pairs, two neighbouring inputs of one row at
-// an even column.  x: the element offset from image n0's channel 0 (kOut: zeros); y: the first one's
-// position plus one in bits 0-15, bits 30 and 31 whether the first and the second are staged.
-__device__ __forceinline__ uint2 pair_entry(const TcParams& p, const Unit& U, int m, int n0) {
+// Entry m of a unit's table of copies: VEC inputs of one row from a column that is a multiple of VEC.
+// x: their element offset from image n0's channel 0 (kOut: zeros).  y: the first staged position they
+// go to, plus VEC, in bits 0-15, and a bit a value from bit 28 on that says it is staged: VEC
+// neighbouring positions at stride 1; at stride 2 the even and odd columns of VEC / 2 positions (of
+// even rows; bit 27 says the odd row below exists).
+template <int S, int VEC>
+__device__ __forceinline__ uint2 copy_entry(const TcParams& p, const Unit& U, int m, int n0) {
+    constexpr int NP = VEC / S;   // positions of a copy
+    int row = 0, col = 0;
+    if (!p.tw) {                  // flat: from the copy of the window's first position on
+        window_start(p, U, &row, &col);
+        m += col / NP;
+    }
     const int r = (int)fdiv((uint32_t)m, p.d_ppr), j = m - r * p.ppr;
-    int n, y, x, p0;
-    bool w0, w1;
+    int n, y, x, c0, p0;          // x, y in the output grid
     if (p.tw) {
         n = U.n;
         y = U.oy0 + r - 1;
-        x = U.ox0 - 2 + 2 * j;
-        const int c = 2 * j - 1;
-        p0 = r * p.Wp + c;
-        w0 = c >= 0 && c < p.Wp;
-        w1 = c + 1 < p.Wp;
-        if (r >= p.th + 2) {   // the last entry: the two positions after the last row
+        x = ((U.ox0 - 1) & ~(NP - 1)) + NP * j;
+        c0 = x - (U.ox0 - 1);
+        p0 = r * p.Wp + c0;
+        if (S == 1 && r >= p.th + 2) {   // the last entry: the two positions after the last row
             y = -1;
+            c0 = 0;
             p0 = r * p.Wp;
-            w0 = w1 = true;
         }
     } else {
-        int row, col;
-        window_start(p, U, &row, &col);
         row += r;
-        x = 2 * j;
+        x = c0 = NP * j;
         p0 = r * p.Wp + x - col;
-        w0 = p0 >= 0 && p0 < p.P && x < p.Wp;
-        w1 = p0 + 1 >= 0 && p0 + 1 < p.P && x + 1 < p.Wp;
         y = -1;
         n = 0;
         if (row >= 0) {
@@ -430,9 +436,16 @@ __device__ __forceinline__ uint2 pair_entry(const TcParams& p, const Unit& U, in
     }
     uint2 e;
     e.x = kOut;
-    if (n < p.N && y >= 0 && y < p.H && x >= 0 && x < p.W)
-        e.x = ((uint32_t)(n - n0) * (uint32_t)p.C * p.H + (uint32_t)y) * p.W + (uint32_t)x;
-    e.y = (w0 || w1 ? (uint32_t)(p0 + 1) : 0u) | (w0 ? 1u << 30 : 0u) | (w1 ? 1u << 31 : 0u);
+    e.y = 0;
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+        if (c0 + a >= 0 && c0 + a < p.Wp && p0 + a >= 0 && p0 + a < p.P) e.y |= (S == 1 ? 1u : 3u) << (28 + S * a);
+    }
+    if (e.y) e.y |= (uint32_t)(p0 + VEC);
+    if (n < p.N && y >= 0 && y < p.Ho && x >= 0 && x * S < p.W) {
+        e.x = ((uint32_t)(n - n0) * (uint32_t)p.C * p.H + (uint32_t)(y * S)) * p.W + (uint32_t)(x * S);
+        if (S == 2 && 2 * y + 1 < p.H) e.y |= 1u << 27;
+    }
     return e;
 }
 
@@ -440,20 +453,20 @@ __device__ __forceinline__ uint2 pair_entry(const TcParams& p, const Unit& U, in
 // asynchronously to its own column of a ring in shared memory (neighbouring lanes neighbouring
 // addresses), and RING - 1 items later splits them and stores 16 bytes of hi and of lo a position.
 // The copies run ahead over blocks and units.  What held this part was first the latency of its loads
-// (two items ahead in registers: 0.85 clocks a value), then the number of copies, a warp's copy of 4
-// bytes a lane taking some 16 clocks: so with PAIR (rows of even length, inputs aligned to two values)
-// a copy brings two values, two neighbouring positions at stride 1, a position's even and odd column
-// at stride 2 (256 -> 256, 28x28 to 14x14, batch 64: 64 -> 51 us).  fp16 inputs are exact: their 16
-// bits go to the stage as they are; the copy has no 2-byte form, so they come in pairs only.
-template <int S, typename T, bool PAIR>
+// (two items ahead in registers: 0.85 clocks a value), then the number of copies, a warp's copy
+// taking some 16 clocks whether of 4 or 8 bytes a lane: so where rows are a multiple of VEC inputs
+// and x is aligned to them a copy brings VEC values (256 -> 256, 28x28 to 14x14, batch 64: 64 us with
+// one, 51 with two).  fp16 inputs are exact: their 16 bits go to the stage as they are; the copy has no
+// 2-byte form, so VEC is 2 or 4.
+template <int S, typename T, int VEC>
 __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
                                             volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
     constexpr bool F32 = sizeof(T) == 4;
-    static_assert(F32 || PAIR, "fp16 values are copied in pairs");
+    static_assert(F32 || VEC > 1, "fp16 values are copied in pairs at least");
     constexpr int HL = F32 ? 2 : 1;
-    constexpr int V = PAIR ? 2 : 1;                  // values of a channel in an item
-    constexpr int WV = F32 ? V : 1;                  // words they take
-    constexpr int RING = WV == 2 ? kRingPair : kRing;
+    constexpr int V = VEC;                           // values of a channel in an item
+    constexpr int WV = F32 ? V : V / 2;              // words they take
+    constexpr int RING = ring_of(WV);
     constexpr int SLOT = (8 * WV + 1) * kProducers;  // words of a ring slot: the values, where they go
     const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
     const uint32_t HW = (uint32_t)p.H * p.W, HWB = HW * (uint32_t)sizeof(T);
@@ -461,39 +474,38 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
     uint2* table2 = reinterpret_cast<uint2*>(table);
     const int steps = (p.items + kProducers - 1) / kProducers;
     float* ring = reinterpret_cast<float*>(smem + p.ring_off);
-    const uint32_t second = S == 1 ? 16u : 2u * HL * p.plane;   // an item's second value: next position, or odd columns' plane
+    // byte offset in the stage of an item's value a: positions side by side, at stride 2 the odd
+    // columns in a plane of their own
+    auto place = [&](int a) { return S == 1 ? 16u * a : 16u * (a >> 1) + (a & 1) * (2u * HL * p.plane); };
     // item i of a unit, from a table entry: whether its inputs exist, their offset, and where it goes
-    // (byte offset in the stage; bits 30 and 31: the first and second value are staged)
+    // (byte offset in the stage plus 16 VEC; from bit 28 on: the values that are staged)
     auto decode = [&](int i, auto&& entry, uint32_t* off, uint32_t* dst) {
-        if (i >= p.items) {
-            *dst = 0;
-            return false;
-        }
-        if constexpr (S == 1 && PAIR) {
-            const int k = i >= p.n_entries ? 1 : 0;
+        *dst = 0;
+        if (i >= p.items) return false;
+        if constexpr (VEC > 1) {
+            const int k = (int)fdiv((uint32_t)i, p.d_p);   // channel half, at stride 2 + 2 (odd rows)
             const uint2 e = entry(i - k * p.n_entries);
-            *off = e.x + (k ? 8u * HW : 0u);
-            const uint32_t p1 = e.y & 0xFFFFu;   // position + 1
-            *dst = (e.y & 0xC0000000u) | (p1 * 16u + (uint32_t)k * p.plane);
-            return e.x != kOut;
+            const int odd_row = S == 2 ? k >> 1 : 0;
+            *off = e.x + ((k & 1) ? 8u * HW : 0u) + (uint32_t)odd_row * p.W;
+            if (e.y) *dst = (e.y & 0xF0000000u) | ((e.y & 0xFFFFu) * 16u + (uint32_t)(odd_row * 4 * HL + (k & 1)) * p.plane);
+            return e.x != kOut && (!odd_row || (e.y & (1u << 27)));
         } else {
             const int k = (int)fdiv((uint32_t)i, p.d_p);
             const int pos = i - k * p.P;
             const uint32_t t = entry(pos).x;
             bool in = t != kOut;
             *off = (t >> 2) + ((k & 1) ? 8u * HW : 0u);
-            // planes at stride 2: 2 (odd rows) + (odd columns)
-            const int odd_row = PAIR ? k >> 1 : k >> 2, odd_col = PAIR ? 0 : (k >> 1) & 1;
+            const int odd_row = k >> 2, odd_col = (k >> 1) & 1;
             if constexpr (S == 2) {
                 in = in && (!odd_col || (t & 1u)) && (!odd_row || (t & 2u));
                 *off += (uint32_t)odd_row * p.W + (uint32_t)odd_col;
             }
             const int pl = S == 1 ? 0 : 2 * odd_row + odd_col;
-            *dst = (PAIR ? 0xC0000000u : 0x40000000u) | ((uint32_t)(pl * 2 * HL + (k & 1)) * p.plane + (uint32_t)(pos + 1) * 16u);
+            *dst = 0x10000000u | ((uint32_t)(pl * 2 * HL + (k & 1)) * p.plane + (uint32_t)(pos + 1) * 16u);
             return in;
         }
     };
-    auto channel_of = [&](int i) { return S == 1 && PAIR ? (i >= p.n_entries ? 8 : 0) : (int)(fdiv((uint32_t)i, p.d_p) & 1u) * 8; };
+    auto channel_of = [&](int i) { return (int)(fdiv((uint32_t)i, p.d_p) & 1u) * 8; };
     int kexp = 0;
     Stage sg;
     // the copies' cursor: unit, block, step, slot
@@ -506,7 +518,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                 const int n0 = first_image(p, U);
                 bar_or<1, kProducers>(false);
                 for (int i = tid; i < p.n_entries; i += kProducers) {
-                    if constexpr (S == 1 && PAIR) table2[i] = pair_entry(p, U, i, n0);
+                    if constexpr (VEC > 1) table2[i] = copy_entry<S, VEC>(p, U, i, n0);
                     else table[i] = window_entry<S>(p, U, i, n0);
                 }
                 bar_or<1, kProducers>(false);
@@ -517,7 +529,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
             const int i = tid + ig * kProducers;
             uint32_t off, dst;
             const bool in = decode(i, [&](int m) {
-                if constexpr (S == 1 && PAIR) return table2[m];
+                if constexpr (VEC > 1) return table2[m];
                 else return make_uint2(table[m], 0u);
             }, &off, &dst);
             float* slot = ring + islot * SLOT;
@@ -555,20 +567,20 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
         const Unit U = unit_of(p, u, rank);
         for (int cb = U.cb0; cb < U.cb1; ++cb) {
             const bool ok = sg.e < p.xs || wait_bar(xempty + 8 * sg.s, (sg.ph & 1) ^ 1, p, abort_flag, kErrSpace);
-            unsigned char* st = smem + p.x_off + (size_t)sg.s * p.x_stage - 16;   // positions are one too high
+            unsigned char* st = smem + p.x_off + (size_t)sg.s * p.x_stage - 16 * VEC;
             uint32_t mn = 0xFFFFFFFFu, bad = 0;
             __half2 hmx = __half2half2(__ushort_as_half(0));
             float scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
             auto split = [&](const float (&v)[WV][8], uint32_t dst) {
 #pragma unroll
                 for (int a = 0; a < V; ++a) {
-                    if (!(dst & (0x40000000u << a))) continue;
-                    unsigned char* d = st + (dst & 0x3FFFFFFFu) + a * second;
-                    if constexpr (!F32) {   // a word holds a channel's two values
+                    if (!(dst & (0x10000000u << a))) continue;
+                    unsigned char* d = st + (dst & 0x0FFFFFFFu) + place(a);
+                    if constexpr (!F32) {   // a word holds two values of a channel
                         uint32_t w[4];
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            w[j] = __byte_perm(__float_as_uint(v[0][2 * j]), __float_as_uint(v[0][2 * j + 1]), a ? 0x7632 : 0x5410);
+                            w[j] = __byte_perm(__float_as_uint(v[a / 2 % WV][2 * j]), __float_as_uint(v[a / 2 % WV][2 * j + 1]), a & 1 ? 0x7632 : 0x5410);
                             bad |= ((w[j] & 0x7C007C00u) + 0x04000400u) & 0x80008000u;   // exponent 31: not finite
                         }
                         *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -591,7 +603,13 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                 const uint32_t dst = reinterpret_cast<const uint32_t*>(from)[8 * WV * kProducers + tid];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    if constexpr (WV == 2) {
+                    if constexpr (WV == 4) {
+                        const float4 t = *reinterpret_cast<const float4*>(from + 4 * (j * kProducers + tid));
+                        v[0][j] = t.x;
+                        v[1 % WV][j] = t.y;
+                        v[2 % WV][j] = t.z;
+                        v[3 % WV][j] = t.w;
+                    } else if constexpr (WV == 2) {
                         const float2 t = *reinterpret_cast<const float2*>(from + 2 * (j * kProducers + tid));
                         v[0][j] = t.x;
                         v[WV - 1][j] = t.y;
@@ -620,7 +638,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                     auto again = [&](int i, float (&v)[V][8]) {
                         uint32_t off, dst;
                         const bool in = decode(i, [&](int m) {
-                            if constexpr (S == 1 && PAIR) return pair_entry(p, U, m, n0);
+                            if constexpr (VEC > 1) return copy_entry<S, VEC>(p, U, m, n0);
                             else return make_uint2(window_entry<S>(p, U, m, n0), 0u);
                         }, &off, &dst);
                         const int nch = in ? p.C - cb * 16 - channel_of(i) : 0;
@@ -635,7 +653,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                     for (int g = 0; g < steps; ++g) {
                         const uint32_t dst = again(tid + g * kProducers, v);
                         for (int a = 0; a < V; ++a)
-                            if (dst & (0x40000000u << a))
+                            if (dst & (0x10000000u << a))
                                 for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[a][j]));
                     }
                     if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
@@ -1022,8 +1040,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
-            if (p.ppr) produce_async<S, T, true>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
-            else if constexpr (HL == 2) produce_async<S, T, false>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            else if (p.vec == 2) produce_async<S, T, 2>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            else if constexpr (HL == 2) produce_async<S, T, 1>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             asm volatile("cp.async.wait_all;" ::: "memory");   // after a timeout: nothing in flight at the exit
         } else if (warp == kLoaderWarp) {
@@ -1285,10 +1304,10 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
     bool have = false;
     // Tiles of 128, 256 or 512 positions: flat (no pool), or rectangles of a k-th of the width and as
     // many rows as fit, evened out
-    for (int i = 0; i < 3 * 17; ++i) {
-        const int k = i % 17;
+    for (int i = 0; i < 3 * 10; ++i) {
+        const int k = i % 10 < 7 ? i % 10 : (i % 10 == 9 ? 16 : 4 * (i % 10) - 20);   // 0 ... 6, 8, 12, 16
         TensorPlan c = pl;
-        c.MT = 1 << (i / 17);
+        c.MT = 1 << (i / 10);
         if (c.MT > mt_max) break;
         if (pool && k == 0) continue;
         const int M = 128 * c.MT;
@@ -1324,6 +1343,7 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         }
         if (tiles >= INT_MAX / 4) continue;
         c.tiles = (int)((tiles + 1) / 2);
+        if (c.P >= 0xFFFF) continue;
         // the MMAs read 128 MT rows from every tap's offset on, staged or not
         const int rows = S == 1 ? M + 2 * c.Wp + 2 : M + c.Wp + 1;
         c.plane = (unsigned)align_up((size_t)std::max(rows, c.P) * 16, 128);
@@ -1331,69 +1351,65 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         // pooling: 32, 16 or 8 filters of a tile's outputs at an even row pitch
         const size_t pool_bytes = pool ? (size_t)32 / c.MT * c.th * ((c.tw + 1) & ~1) * 4 : 0;
         c.tab_off = (unsigned)(kHeadBytes + align_up(pool_bytes, 16));
-        // items of a block: pairs of pixels where rows are even (and x is aligned to a pair:
-        // tensor_launch) unless that takes more rounds of the staging threads (fp16: as many); ppr is
-        // the pairs of a staged row, 0 with single pixels
-        const auto rounds_of = [](int n) { return (n + kProducers - 1) / kProducers; };
-        c.n_entries = c.P;
-        c.items = 2 * c.P * (S == 1 ? 1 : 4);
-        if (W % 2 == 0) {
-            const int ppr = S == 2 ? 2 : (c.tw ? (c.Wp + 2) / 2 : W / 2 + 1);
-            const int entries = S == 2 ? c.P : (c.tw ? (c.th + 2) * ppr + 1 : ((c.P + c.Wp - 1) / c.Wp + 1) * ppr);
-            const int items = S == 2 ? 4 * c.P : 2 * entries;
-            if (rounds_of(items) < rounds_of(c.items) + (es == 4 ? 1 : 0)) {
-                c.ppr = ppr;
-                c.n_entries = entries;
-                c.items = items;
-            }
-        }
-        if (c.P >= 0xFFFF) continue;
-        c.ring_off = (unsigned)align_up(c.tab_off + std::max<size_t>(4 * (size_t)c.P, 8 * (size_t)c.n_entries), 128);
-        c.x_off = c.ring_off + (es == 4 ? std::max(kRing * 9, kRingPair * 17) : kRing * 9) * kProducers * 4;
-        if (c.x_off >= kSmemMax) continue;
-        const size_t left = kSmemMax - c.x_off;
-        // three input stages with two blocks' weights, else two with at least a block's and a row
-        c.xs = 0;
-        for (int xs = 3; xs >= 2 && !c.xs; --xs) {
-            const int hs = xs == 3 ? 6 : 4, ls = 2;
-            if ((size_t)xs * c.x_stage + (size_t)(hs + ls) * c.w_slot > left) continue;
-            c.xs = xs;
-            const int slots = (int)std::min<size_t>(10, (left - (size_t)xs * c.x_stage) / c.w_slot);
-            c.hs = std::min(6, slots - 2);
-            c.ls = std::min(4, slots - c.hs);
-        }
-        if (!c.xs) continue;
-        c.h_off = c.x_off + c.xs * c.x_stage;
-        c.l_off = c.h_off + c.hs * c.w_slot;
-        c.smem = c.l_off + (size_t)c.ls * c.w_slot;
         const long long units1 = (long long)c.tiles * c.n_fchunks, pairs = sms / 2;
-        // clocks of a 16-channel block: its MMAs, and the rounds of staging that do not hide behind
-        // them (fitted to 19 layers with every tile each can take: within 10 %); rows of few outputs
-        // cost partial sectors, as 2.5 / width of the whole
         const double mma = 9.0 * (HL + 1) * c.MT * std::max(c.NC / 2.0, 32.0 + c.NC / 8.0) + 200.0;
-        const int rounds = rounds_of(c.items);
-        const double stage = es == 2 ? mma + 700.0 * std::max(0.0, rounds - (S == 1 ? 1.0 : 0.0))
-                             : c.ppr ? mma + 1000.0 * std::max(0.0, rounds - mma / 1900.0)
-                                     : mma + 600.0 * std::max(0.0, rounds - mma / 1000.0);
-        const double narrow = 1.0 + 2.5 / (c.tw ? c.tw : Wo);
-        for (int ks = 1; ks <= c.n_cb; ++ks) {
-            const int cbs = (c.n_cb + ks - 1) / ks;
-            if ((c.n_cb + cbs - 1) / cbs != ks) continue;
-            if (ks > 1 && (size_t)ks * out_bytes > ws_bytes) break;
-            if (units1 * ks > INT_MAX / 2) break;
-            const long long waves = (units1 * ks + pairs - 1) / pairs;
-            const double stores = 128.0 * c.MT * c.NC * (ks > 1 ? 4 : es) / 10.0;
-            double t = waves * (std::max(cbs * stage, stores) + 1500.0) * narrow + 6000.0;
-            if (ks > 1) t += 4000.0 + (double)ks * out_bytes / 2000.0;
-            if (!have || t < best) {
-                have = true;
-                best = t;
-                *out = c;
-                out->KS = ks;
-                out->cb_split = cbs;
-                out->units = units1 * ks;
-                out->ws_bytes = ks > 1 ? (size_t)ks * out_bytes : 0;
-                out->clocks = t;
+        // a copy brings one, two or four values, where rows are a multiple of them (and x is aligned:
+        // tensor_launch)
+        for (int vec = 1; vec <= 4 && W % vec == 0; vec *= 2) {
+            c.vec = vec;
+            const int np = std::max(1, vec / S);   // positions of a copy
+            c.ppr = c.tw ? (c.Wp + 2 * (np - 1)) / np : Wo / np + 1;
+            // flat tiles: the copies from that of the first position to that of the last, P - 1 further
+            c.n_entries = np == 1 && !c.tw ? c.P
+                          : vec == 1       ? c.P
+                          : c.tw           ? (S == 1 ? (c.th + 2) * c.ppr + 1 : (c.th + 1) * c.ppr)
+                                           : (c.P - 1) / c.Wp * c.ppr + (c.P - 1) % c.Wp / np + 3;
+            c.items = vec == 1 ? 2 * c.P * (S == 1 ? 1 : 4) : 2 * S * c.n_entries;
+            c.ring_off = (unsigned)align_up(c.tab_off + std::max<size_t>(4 * (size_t)c.P, 8 * (size_t)c.n_entries), 128);
+            const int words = es == 4 ? vec : std::max(1, vec / 2);
+            c.x_off = c.ring_off + std::max(ring_of(1) * 9, ring_of(words) * (8 * words + 1)) * kProducers * 4;
+            if (c.x_off >= kSmemMax) continue;
+            const size_t left = kSmemMax - c.x_off;
+            // three input stages with two blocks' weights, else two with at least a block's and a row
+            c.xs = 0;
+            for (int xs = 3; xs >= 2 && !c.xs; --xs) {
+                const int hs = xs == 3 ? 6 : 4, ls = 2;
+                if ((size_t)xs * c.x_stage + (size_t)(hs + ls) * c.w_slot > left) continue;
+                c.xs = xs;
+                const int slots = (int)std::min<size_t>(10, (left - (size_t)xs * c.x_stage) / c.w_slot);
+                c.ls = slots < 7 ? 2 : (slots < 10 ? 3 : 4);
+                c.hs = slots - c.ls;
+            }
+            if (!c.xs) continue;
+            c.h_off = c.x_off + c.xs * c.x_stage;
+            c.l_off = c.h_off + c.hs * c.w_slot;
+            c.smem = c.l_off + (size_t)c.ls * c.w_slot;
+            // clocks of a 16-channel block: its MMAs, and what of its staging does not hide behind
+            // them, by rounds of the staging threads; of a unit: its blocks or its stores.  Fitted to
+            // 24 layers with every tile, copy and split each can take (849 points, 5 % rms weighted
+            // towards the fast ones; the choice is 1.5 % from the best on average).
+            static const double kRound[2][3] = {{840.0, 1280.0, 1920.0}, {840.0, 945.0, 1030.0}};   // fp32, fp16
+            const int rounds = (c.items + kProducers - 1) / kProducers;
+            const double staging = rounds * kRound[es == 2][vec == 1 ? 0 : vec / 2];
+            const double stage = (mma + std::max(0.0, staging - 0.64 * mma)) * (c.hs + c.ls < 8 ? 1.09 : 1.0);
+            for (int ks = 1; ks <= c.n_cb && (ks == 1 || units1 * ks <= 2 * pairs); ++ks) {
+                const int cbs = (c.n_cb + ks - 1) / ks;
+                if ((c.n_cb + cbs - 1) / cbs != ks) continue;
+                if (ks > 1 && (size_t)ks * out_bytes > ws_bytes) break;
+                const long long waves = (units1 * ks + pairs - 1) / pairs;
+                const double stores = 128.0 * c.MT * c.NC * (ks > 1 ? 4 : es) / 10.0;
+                double t = waves * (std::max(cbs * stage, stores) + 6000.0) * (1.0 + 0.5 / (c.tw ? c.tw : Wo)) + 6000.0;
+                if (ks > 1) t += 4000.0 + (double)ks * out_bytes / 2000.0;
+                if (!have || t < best) {
+                    have = true;
+                    best = t;
+                    *out = c;
+                    out->KS = ks;
+                    out->cb_split = cbs;
+                    out->units = units1 * ks;
+                    out->ws_bytes = ks > 1 ? (size_t)ks * out_bytes : 0;
+                    out->clocks = t;
+                }
             }
         }
     }
@@ -1424,6 +1440,7 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.Ip = pl.Ip;
     p.mstep = pl.mstep;
     p.P = pl.P;
+    p.vec = pl.vec;
     p.ppr = pl.ppr;
     p.n_entries = pl.n_entries;
     p.items = pl.items;
@@ -1437,7 +1454,7 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.n_units = (int)pl.units;
     p.d_ip = fast_div((uint32_t)pl.Ip);
     p.d_wp = fast_div((uint32_t)pl.Wp);
-    p.d_p = fast_div((uint32_t)p.P);
+    p.d_p = fast_div((uint32_t)(pl.vec > 1 ? pl.n_entries : pl.P));
     p.d_ppr = fast_div((uint32_t)std::max(2, pl.ppr));
     p.ws = static_cast<float*>(c.ws);
     p.ws_stride = (size_t)c.N * L->cout * c.Ho * c.Wo;
@@ -1453,10 +1470,11 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.x_off = pl.x_off;
     p.h_off = pl.h_off;
     p.l_off = pl.l_off;
-    if (pl.ppr && reinterpret_cast<uintptr_t>(c.x) % (2 * (size_t)c.es) != 0) {   // single pixels after all
-        p.ppr = 0;
+    if (pl.vec > 1 && reinterpret_cast<uintptr_t>(c.x) % (pl.vec * (size_t)c.es) != 0) {   // single pixels after all
+        p.vec = 1;
         p.n_entries = pl.P;
         p.items = 2 * pl.P * (L->stride == 1 ? 1 : 4);
+        p.d_p = fast_div((uint32_t)p.P);
     }
     TcKernel k;
     if (L->stride == 1) k = c.es == 4 ? pick<1, float>(pl.MT, pl.smem) : pick<1, __half>(pl.MT, pl.smem);

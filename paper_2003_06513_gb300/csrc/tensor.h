@@ -17,7 +17,7 @@ struct TensorPlan {
     long long Q = 0;        // flat tiles: positions of the padded output grid
     int mstep = 0;          // flat tiles: positions a tile advances
     int P = 0;              // positions a tile stages
-    int ppr = 0, n_entries = 0, items = 0;   // pixel pairs of a staged row (0: single pixels), table, items
+    int vec = 1, ppr = 0, n_entries = 0, items = 0;   // values a copy, copies of a staged row, table, items
     int tw = 0, th = 0, tiles_x = 0, tiles_y = 0;   // rectangles of outputs (tw 0: flat tiles)
     int tiles = 0, n_fchunks = 0;   // tiles: pairs of position tiles, one per CTA of a pair
     long long units = 0;
