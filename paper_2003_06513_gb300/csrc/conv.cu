@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cmath>
 #include <cstdlib>
 #include <cstdint>
 #include <cstring>
@@ -2648,17 +2649,29 @@ int make_plan_uncached(const pp_layer* L, int N, int H, int W, size_t ws_avail, 
 double shift_gain(double kept_per_channel) { return std::min(1.0, 0.82 + 0.0225 * kept_per_channel); }
 
 // Whether a call takes the tensor-core kernel: where its estimate is the lower one, and for fp32 only
-// where its rounding error is no larger.  The FFMA kernel's error grows with the number of products
-// it adds one after the other (1.1e-7 of the result at 77, 2.2e-7 at 307, 2.7e-7 at 614; 7e-8 at
-// 12), the tensor cores' starts at 0.9e-7 (the fp16 pairs) and grows slower (1.25e-7 at 307, 1.45e-7
-// at 614).
+// where its rounding error is no larger.  Squared errors against 64 bits, in units of (1e-7 of the
+// result)^2, fitted to VGG-16's layers at batch 1 and 32:
+//   FFMA           0.06 + 0.0137 products / KS + 0.036 KS     (77 products 1.1e-7, 307 2.2e-7, 614 in
+//                                                               32 splits 1.2e-7)
+//   tensor cores   1.0 + 0.033 blocks + 0.058 log2 KS         (0.84 for 1.0 with the lo products; the
+//                                                               pairs alone are 0.7e-7)
+// Three products need 72 products a split instead of the formula (measured 0.9e-7 against 1.1e-7
+// there), and four at least 8, below which the formula says too much of the FFMA kernel.
 bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int es) {
     const double products = 4.0 * L->beta / L->cout;
-    if (es == 4 && products < 72.0 * pl.KS) return false;
+    if (es == 4 && !pl.tc.ll && products < 72.0 * pl.KS) return false;
+    if (es == 4 && pl.tc.ll) {
+        const double ffma = 0.06 + 0.0137 * products / pl.KS + 0.036 * (pl.KS > 1 ? pl.KS : 0);
+        const double tensor = 0.84 + 0.033 * pl.tc.cb_split + 0.058 * std::log2((double)pl.tc.KS);
+        if (products < 8.0 * pl.KS || tensor > ffma) return false;
+    }
     if (!L->fast) return true;
     const double flop = 8.0 * L->beta * (double)N * Ho * Wo;
     const double rate = (es == 4 ? 28e6 : 24e6) * (L->stride == 2 ? 0.5 : 1.0);   // FLOP a microsecond
-    return pl.tc.clocks / 1900.0 + 3.0 < 0.95 * (flop / rate + 8.0);
+    // microseconds beside the contraction: the launch, with a split its partial sums and reduction
+    // (VGG-16 at batch 1: 19 with 3 splits, 28 with 32)
+    const double other = pl.KS > 1 ? 14.0 + 0.3 * pl.KS : 8.0;
+    return pl.tc.clocks / 1900.0 + 3.0 < 0.95 * (flop / rate + other);
 }
 
 int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out, int pool = 0,
@@ -2691,8 +2704,11 @@ int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out
             cs * shift_gain(kpc) < cost)
             pl = ps;
     }
-    pl.tensor = tensor_plan(L, N, H, W, pool, es, ws_avail, sm_count(), &pl.tc) &&
-                tensor_wins(L, pl, N, (H - 1) / L->stride + 1, (W - 1) / L->stride + 1, es);
+    // fp32: with three products where that rounds no more than the FFMA kernel's plan, else with four
+    const int Ho = (H - 1) / L->stride + 1, Wo = (W - 1) / L->stride + 1;
+    for (int ll = 0; ll < (es == 4 ? 2 : 1) && !pl.tensor; ++ll)
+        pl.tensor = tensor_plan(L, N, H, W, pool, es, ws_avail, sm_count(), &pl.tc, ll) &&
+                    tensor_wins(L, pl, N, Ho, Wo, es);
     std::lock_guard<std::mutex> g(cache->mu);
     if (cache->plans.size() >= 256) cache->plans.clear();
     cache->plans[key] = pl;
@@ -2703,8 +2719,12 @@ int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out
 // Sum the KS partial planes in split order, + bias, ReLU, round to the output type.  A thread
 // issues the loads of 8 splits before it adds them, so that many loads are in flight; with
 // `quads` (large outputs, a multiple of 4 elements, 16-byte aligned workspace) it takes 4
-// consecutive elements, one 16-byte load per split.  Each element is still summed in split order
-// (the result is that of a plain loop over the splits).
+// consecutive elements, one 16-byte load per split.  Eight splits are summed pairwise before they are
+// added (a fixed order, the same for every path): of 32 partial sums added one after the other the
+// rounding alone was 1e-7 of the result.
+__device__ __forceinline__ float sum8(float a, float b, float c, float d, float e, float f, float g, float h) {
+    return ((a + b) + (c + d)) + ((e + f) + (g + h));
+}
 template <typename T>
 __global__ void splitk_reduce(const float* __restrict__ ws, T* __restrict__ y, const float* __restrict__ bias,
                               int KS, size_t stride, int Cout, int HoWo, int relu, int quads) {
@@ -2725,13 +2745,10 @@ __global__ void splitk_reduce(const float* __restrict__ ws, T* __restrict__ y, c
                 float4 t[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) t[j] = w4[(size_t)(k + j) * s4];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    a.x += t[j].x;
-                    a.y += t[j].y;
-                    a.z += t[j].z;
-                    a.w += t[j].w;
-                }
+                a.x += sum8(t[0].x, t[1].x, t[2].x, t[3].x, t[4].x, t[5].x, t[6].x, t[7].x);
+                a.y += sum8(t[0].y, t[1].y, t[2].y, t[3].y, t[4].y, t[5].y, t[6].y, t[7].y);
+                a.z += sum8(t[0].z, t[1].z, t[2].z, t[3].z, t[4].z, t[5].z, t[6].z, t[7].z);
+                a.w += sum8(t[0].w, t[1].w, t[2].w, t[3].w, t[4].w, t[5].w, t[6].w, t[7].w);
             }
             for (; k < KS; ++k) {
                 const float4 t = w4[(size_t)k * s4];
@@ -2753,8 +2770,7 @@ __global__ void splitk_reduce(const float* __restrict__ ws, T* __restrict__ y, c
                 float t[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) t[j] = ws[(size_t)(k + j) * stride + q];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) a += t[j];
+                a += sum8(t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7]);
             }
             for (; k < KS; ++k) a += ws[(size_t)k * stride + q];
             v[0] = a;
@@ -2805,9 +2821,7 @@ __global__ void splitk_reduce_pool(const float* __restrict__ ws, T* __restrict__
 #pragma unroll
                 for (int j = 0; j < 4; ++j) t[kk][j] = ws[(size_t)(k + kk) * stride + base + off[j]];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) q[j] += t[kk][j];
+            for (int j = 0; j < 4; ++j) q[j] += (t[0][j] + t[1][j]) + (t[2][j] + t[3][j]);
         }
         for (; k < KS; ++k) {
 #pragma unroll

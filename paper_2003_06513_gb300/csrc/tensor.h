@@ -13,6 +13,7 @@ struct TensorPlan {
     int NC = 0;             // filters per unit (a multiple of 16)
     int KS = 1;             // input-channel splits (KS > 1: fp32 partial sums in the workspace)
     int n_cb = 0, cb_split = 0;   // 16-channel blocks, blocks per split
+    int ll = 0;             // fp32: the products of the lo parts too
     int Wp = 0, Ip = 0;     // position pitch of a row, of an image (flat tiles)
     long long Q = 0;        // flat tiles: positions of the padded output grid
     int mstep = 0;          // flat tiles: positions a tile advances
@@ -46,7 +47,9 @@ struct TensorCall {
 #endif
 
 // Plan of a call, or false where the tensor-core kernel does not take it.
-bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_t ws_bytes, int sms, TensorPlan* out);
+// ll (fp32): with the products of the lo parts, a third more work for less rounding.
+bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_t ws_bytes, int sms, TensorPlan* out,
+                 int ll = 0);
 #ifdef __CUDACC__
 cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl);
 // Builds the tensor-core weights from the bound device image.

@@ -103,17 +103,23 @@ def test_tensor_kernel_matches_oracle(case):
     _check(y, x, W, b, keep, stride, pool, io, idx=[0, n // 2, n - 1])
 
 
-def test_tensor_split_of_the_input_channels():
-    """Few tiles and a workspace: partial sums per channel range, added by the reduction."""
-    layer, W, b = _layer(256, 512, 1.0, 1, 3)
-    x = WL.activations((6, 512, 14, 14), 4, relu=True)
+@pytest.mark.parametrize("case", [(512, 512, 1, 14, 14, 0.3, False), (512, 512, 1, 28, 28, 0.3, True),
+                                  (256, 256, 4, 14, 14, 0.4, False), (128, 256, 2, 16, 17, 0.5, False)])
+def test_tensor_split_of_the_input_channels(case):
+    """Few tiles and a workspace: partial sums per channel range, with the products of the lo parts
+    (the CUDA-core plan, itself split, rounds less than three products do), added by the reduction;
+    the same result again."""
+    cout, cin, n, h, w, keep, pool = case
+    layer, W, b = _layer(cout, cin, keep, 1, 3 + h)
+    x = WL.activations((n, cin, h, w), 4, relu=True)
     xt = torch.from_numpy(x).cuda()
-    ws = torch.full((1 << 22,), float("nan"), device="cuda")
-    plan = layer.tensor_plan(xt.shape, ws.numel() * 4)
-    if not plan["tensor"]:
-        pytest.skip("this shape takes the CUDA-core kernel")
-    y = layer.conv(xt, torch.from_numpy(b).cuda(), True, workspace=ws)
-    _check(y, x, W, b, 1.0, 1, False, "f32")
+    ws = torch.full((1 << 23,), float("nan"), device="cuda")
+    plan = layer.tensor_plan(xt.shape, ws.numel() * 4, pool)
+    assert plan["tensor"] == 1 and plan["splits"] > 1
+    bt = torch.from_numpy(b).cuda()
+    y = layer.conv(xt, bt, True, workspace=ws, pool2x2=pool)
+    _check(y, x, W, b, keep, 1, pool, "f32")
+    assert torch.equal(layer.conv(xt, bt, True, workspace=ws, pool2x2=pool), y)
 
 
 def test_tensor_kernel_other_pattern_library():
