@@ -9,9 +9,10 @@ N(0,1) images (the paper's trained networks and ImageNet images are not availabl
 
 Prints one JSON line (rank 0).  `value` is images/s over all ranks (each rank runs its own
 batch: weak scaling, no collective in the data path).  Extra keys:
-  roofline      the dominant kernel (pconv_tm) against the FP32 CUDA-core peak
-                (SMs x 128 lanes x 2 FLOP x max SM clock), from CUDA events around each of its
-                launches inside the timed region;
+  roofline      the convolution kernels' useful FLOP (kept weights) against the FP32 CUDA-core
+                peak measured on this GPU, from CUDA events around each of their launches inside the
+                timed region; its `tensor` entry counts what the tensor-core layers issue (three fp16
+                products of the dense contraction) against the measured bf16 peak;
   e2e           the same metric with every step's input batch copied from pinned host memory
                 and its final feature map copied back inside the timed region (the copies on a
                 second stream, double-buffered, overlapping the neighbouring steps' compute);
@@ -314,22 +315,32 @@ def hbm_peak():
         return 6.8e12, "fallback"
 
 
+def tensor_peak():
+    """Measured dense bf16 throughput of this kind of GPU in TFLOP/s (cuBLAS, burst), or None."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"])
+    except Exception:
+        return None
+
+
 def kernel_sources_sha256():
-    """Hash of the kernel's sources: conv.cu and the channel loop its generator emits."""
+    """Hash of the kernels' sources: tensor.cu, conv.cu and the channel loop its generator emits."""
     import importlib.util
     csrc = os.path.join(ROOT, "paper_2003_06513_gb300", "csrc")
     spec = importlib.util.spec_from_file_location("gen_dispatch", os.path.join(csrc, "gen_dispatch.py"))
     gen = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(gen)
     h = hashlib.sha256()
-    with open(os.path.join(csrc, "conv.cu"), "rb") as f:
-        h.update(f.read())
+    for name in ("tensor.cu", "conv.cu"):
+        with open(os.path.join(csrc, name), "rb") as f:
+            h.update(f.read())
     h.update(gen.generate().encode())
     return h.hexdigest()
 
 
 def traffic_record():
-    """Per-launch DRAM bytes of pconv_tm on this workload from the committed ncu summary, or
+    """Per-launch DRAM bytes of the kernels on this workload from the committed ncu summary, or
     None when the kernel source changed since the counters were taken."""
     path = os.path.join(ROOT, "profiles", "pconv_tm_vgg16_b32_traffic.txt")
     try:
@@ -433,9 +444,11 @@ def our_arm(args, rank, world, local_rank):
     barrier()
 
     K = args.steps
+    ws_bytes = 0 if workspace is None else workspace.numel() * 4
+    tensor = [lay.tensor_plan(sh, ws_bytes, L.pool_after) for lay, sh, L in zip(packed, in_shapes, layers)]
     launches_per_step = len(layers) + sum(
-        1 for lay, sh in zip(packed, in_shapes)
-        if lay.plan(sh, 0 if workspace is None else workspace.numel() * 4)["splits"] > 1)
+        1 for lay, sh, t, L in zip(packed, in_shapes, tensor, layers)
+        if (t if t["tensor"] else lay.plan(sh, ws_bytes, L.pool_after))["splits"] > 1)
     evs = [[[torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)]
             for _ in layers] for _ in range(K)]
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -530,6 +543,9 @@ def our_arm(args, rank, world, local_rank):
         per_layer_ms = [statistics.median(conv_ms[k][i] for k in range(K)) for i in range(len(layers))]
         tot_conv_ms = sum(statistics.mean(conv_ms[k][i] for k in range(K)) for i in range(len(layers)))
         achieved = sum(flops) / (tot_conv_ms * 1e-3)
+        on_tensor = [i for i, t in enumerate(tensor) if t["tensor"]]
+        issued = sum(3 * 18.0 * layers[i].cin * layers[i].cout * BATCH * layers[i].ho * layers[i].wo for i in on_tensor)
+        issued_ms = sum(statistics.mean(conv_ms[k][i] for k in range(K)) for i in on_tensor)
         roof_ms = sum(max(f / peak, b / hbm) for f, b in zip(flops, bytes_)) * 1e3
         eager_ms = elapsed_ms / K
         ms_step = min(eager_ms, graph_ms)      # the faster of stream launches and graph replay
@@ -543,13 +559,15 @@ def our_arm(args, rank, world, local_rank):
             "config": config_dict(),
             "useful_gflops": world * sum(flops) / (ms_step * 1e-3) / 1e9,
             "network_roofline_frac": roof_ms / tot_conv_ms,
-            "roofline": {"bound": "alu", "kernel": "pconv_tm<1,float,SORT> (+ split reduce)",
+            "roofline": {"bound": "alu", "kernel": f"pconv_tc ({len(on_tensor)} of {len(layers)} layers), pconv_tm",
                          "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s",
                          "frac": achieved / peak, "peak_kind": "measured", "peak_basis": peak_basis,
                          "peak_nominal": peak_nominal / 1e12, "peak_clocks": peak_clocks,
                          "traffic": (trec or {}).get("dram_bytes_per_launch"),
                          "algorithmic_bytes_per_launch": sum(bytes_) / len(bytes_),
-                         "hbm_peak_gbs": hbm / 1e9, "hbm_peak_kind": hbm_kind},
+                         "hbm_peak_gbs": hbm / 1e9, "hbm_peak_kind": hbm_kind,
+                         "tensor": {"issued": issued / max(issued_ms, 1e-9) / 1e9, "peak": tensor_peak(),
+                                    "unit": "TFLOP/s (fp16 products of the dense contraction)"}},
             "timing": {"eager_ms_per_step": eager_ms, "graph_ms_per_step": graph_ms,
                        "value_from": "graph" if graph_ms <= eager_ms else "eager"},
             "per_layer_ms": [round(v, 4) for v in per_layer_ms],

@@ -2650,20 +2650,25 @@ double shift_gain(double kept_per_channel) { return std::min(1.0, 0.82 + 0.0225 
 
 // Whether a call takes the tensor-core kernel: where its estimate is the lower one, and for fp32 only
 // where its rounding error is no larger.  Squared errors against 64 bits, in units of (1e-7 of the
-// result)^2, fitted to VGG-16's layers at batch 1 and 32:
-//   FFMA           0.06 + 0.0137 products / KS + 0.036 KS     (77 products 1.1e-7, 307 2.2e-7, 614 in
-//                                                               32 splits 1.2e-7)
-//   tensor cores   1.0 + 0.033 blocks + 0.058 log2 KS         (0.84 for 1.0 with the lo products; the
-//                                                               pairs alone are 0.7e-7)
-// Three products need 72 products a split instead of the formula (measured 0.9e-7 against 1.1e-7
-// there), and four at least 8, below which the formula says too much of the FFMA kernel.
+// result)^2, fitted to 40 layers on both kernels:
+//   FFMA           0.06 + 0.0137 products / pieces + 0.036 pieces   (77 products 1.1e-7, 307 2.2e-7,
+//                  614 in 32 pieces 1.2e-7), the sum's pieces being the plan's splits, on the balanced
+//                  schedule 1 + SMs / (2 units); 1.1 times that where it is not split
+//   tensor cores   1.0 + 0.033 blocks a split + 0.058 log2 splits + 0.5 (keep - 0.3), 0.84 for 1.0
+//                  with the lo products (the pairs alone are 0.7e-7); 0.25 more without them where
+//                  the FFMA plan has four splits or more, as what is compared is then small
+// Below 13 products a piece the formula says too much of the FFMA kernel.  Over 150 drawn layers of 3
+// to 512 channels the error was above the FFMA kernel's in 3, by 4 % at most, before the last two
+// constants were raised for them.
 bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int es) {
-    const double products = 4.0 * L->beta / L->cout;
-    if (es == 4 && !pl.tc.ll && products < 72.0 * pl.KS) return false;
-    if (es == 4 && pl.tc.ll) {
-        const double ffma = 0.06 + 0.0137 * products / pl.KS + 0.036 * (pl.KS > 1 ? pl.KS : 0);
-        const double tensor = 0.84 + 0.033 * pl.tc.cb_split + 0.058 * std::log2((double)pl.tc.KS);
-        if (products < 8.0 * pl.KS || tensor > ffma) return false;
+    if (es == 4) {
+        const double products = 4.0 * L->beta / L->cout, keep = products / (4.0 * L->cin_g);
+        const double pieces = pl.streamk ? 1.0 + 0.5 * sm_count() / pl.ctas : pl.KS;
+        const double ffma = (0.06 + 0.0137 * products / pieces + 0.036 * (pieces > 1.0 ? pieces : 0.0)) *
+                            (pl.KS > 1 ? 1.0 : 1.1);
+        const double tensor = (pl.tc.ll ? 0.84 : pl.KS >= 4 ? 1.25 : 1.0) + 0.033 * pl.tc.cb_split +
+                              0.058 * std::log2((double)pl.tc.KS) + 0.5 * std::max(0.0, keep - 0.3);
+        if (products < 13.0 * pieces || tensor > ffma) return false;
     }
     if (!L->fast) return true;
     const double flop = 8.0 * L->beta * (double)N * Ho * Wo;

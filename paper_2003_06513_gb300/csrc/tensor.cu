@@ -848,6 +848,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     constexpr int M = 128 * MT;
     constexpr int HL = sizeof(T) == 4 ? 2 : 1;
     constexpr int TCOL = 256 / MT;                // accumulator columns of a 128-position tile
+    constexpr bool LL = HL == 2 && MT == 1;
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
@@ -1129,8 +1130,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                     fence_after();
                     const uint32_t xa = desc_lo(bar0 + p.x_off + (uint32_t)s * p.x_stage, p.plane);
                     const uint32_t d = tbase + 256u * b;
-                    // l_x l_w (times 2^22) where asked for
-                    if (HL == 2 && p.ll) {
+                    // l_x l_w (times 2^22) where asked for (small calls, 128-position tiles)
+                    if (LL && p.ll) {
                         int l1 = lsl, lp1 = lph;
 #pragma unroll
                         for (int r = 0; r < 3; ++r) {
@@ -1169,7 +1170,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
 #pragma unroll
                                 for (int i = 0; i < MT; ++i) {
                                     if (r + c == 0) {
-                                        if (HL == 2 && p.ll) mma<2>(d + TCOL * i, xt + 128u * i, wl + wtap * c, idesc);
+                                        if (LL && p.ll) mma<2>(d + TCOL * i, xt + 128u * i, wl + wtap * c, idesc);
                                         else mma<0>(d + TCOL * i, xt + 128u * i, wl + wtap * c, idesc);
                                     } else {
                                         mma<1>(d + TCOL * i, xt + 128u * i, wl + wtap * c, idesc);
@@ -1342,7 +1343,7 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         const int k = i % 10 < 7 ? i % 10 : (i % 10 == 9 ? 16 : 4 * (i % 10) - 20);   // 0 ... 6, 8, 12, 16
         TensorPlan c = pl;
         c.MT = 1 << (i / 10);
-        if (c.MT > mt_max) break;
+        if (c.MT > (ll ? 1 : mt_max)) break;
         if (pool && k == 0) continue;
         const int M = 128 * c.MT;
         long long tiles;
