@@ -97,7 +97,8 @@ class Layer:
     # ---- device side
     def bind(self, device=None, stream=None) -> "Layer":
         """Copy the device image into a fresh torch buffer on ``device`` and build the tensor-core
-        weights beside it where the layer has them (async on ``stream``)."""
+        weights beside it where the layer has them (on ``stream``; complete on return, so that calls
+        on any stream may follow, unless the stream is being captured)."""
         device = torch.device(device if device is not None else "cuda")
         if device.type != "cuda":
             raise ValueError("the packed image must live in CUDA device memory")
@@ -113,6 +114,8 @@ class Layer:
             _lib.check("pp_bind_tensor", _lib.load().pp_bind_tensor(
                 self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
             self._tensor_buf = buf
+            if not torch.cuda.is_current_stream_capturing():
+                (stream if stream is not None else torch.cuda.current_stream(device)).synchronize()
         return self
 
     def out_shape(self, x_shape) -> tuple:
@@ -168,7 +171,7 @@ class Layer:
         """y = ReLU?(conv3x3(x, W_hat, stride, pad 1) + bias) via pp_conv_ws; with ``pool2x2``
         the 2x2/2 max-pool of that map, fused into the conv (pp_conv_pool_ws)."""
         if self._dev_buf is None:
-            self.bind(x.device)
+            self.bind(x.device, stream)
         dt = _DT.get(x.dtype)
         if not x.is_cuda or dt is None or not x.is_contiguous() or x.dim() != 4:
             raise ValueError("x must be a contiguous 4-d CUDA float32/float16 tensor (NCHW)")
