@@ -169,8 +169,8 @@ int pp_conv(pp_handle h, const void* x, int dtype, int N, int H, int W,
 /* pp_conv with an optional caller-owned DEVICE workspace (16-byte aligned, no overlap with x or
  * y).  When one pass over all input channels gives too few CTAs to fill the GPU (small images),
  * the input channels are cut into KS contiguous ranges; each range's CTAs write fp32 partial
- * sums into the workspace ([KS][N][Cout][Ho][Wo]) and a second kernel adds the ranges in order,
- * adds the bias, applies ReLU and rounds to the output type.  The result is deterministic; it
+ * sums into the workspace ([KS][N][Cout][Ho][Wo]) and a second kernel adds the ranges in a
+ * fixed order, adds the bias, applies ReLU and rounds to the output type.  The result is deterministic; it
  * can differ from the single-pass sum in the last bits (fp32 summation order).  workspace ==
  * NULL or too small for any split means a single pass.  The dense fast path only; other paths
  * ignore the workspace.  Same errors as pp_conv, plus PP_ERR_ALIGN / PP_ERR_BUFFER for the

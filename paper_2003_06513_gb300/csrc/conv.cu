@@ -1,6 +1,8 @@
 // CUDA kernels and launchers of libpatconv (sm_103a): pattern-sparse 3x3 convolution.
 //
-// Dense layers, main kernel pconv_tm<S, T, SORT, SHIFT, SK, DG>:
+// Dense layers whose handle is bound for the tensor cores run there (pconv_tc, tensor.cu) wherever
+// tensor_wins() below says that it is faster and rounds no more.  All others, main kernel
+// pconv_tm<S, T, SORT, SHIFT, SK, DG>:
 //   * a lane owns a 4x4 block of output pixels of one image; a warp owns one filter group (8
 //     filter slots, the "filter kernel reorder" of §3.4), or DG = 2 groups at stride 2, for its
 //     32 blocks; a CTA is 16 / DG warps = WG filter groups x WS spatial warps over one tile;
@@ -30,8 +32,7 @@
 // Depthwise layers (one pattern per channel, HBM-bound): pconv_dw_stream, per-warp bulk-copy
 // pipelines of a persistent CTA per SM (rows, planes and tiles modes) for 16-byte aligned
 // tensors; pconv_depthwise / pconv_depthwise_staged for the rest.  Other pattern libraries:
-// pconv_generic.  The path is a gathered sparse contraction, so it runs on the CUDA-core FFMA
-// pipe.
+// pconv_generic.  The kernels of this file compute on the CUDA cores' FFMA pipe.
 #include <cuda_fp16.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -2721,7 +2722,7 @@ int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out
     return PP_OK;
 }
 
-// Sum the KS partial planes in split order, + bias, ReLU, round to the output type.  A thread
+// Sum the KS partial planes (eight at a time, pairwise), + bias, ReLU, round to the output type.  A thread
 // issues the loads of 8 splits before it adds them, so that many loads are in flight; with
 // `quads` (large outputs, a multiple of 4 elements, 16-byte aligned workspace) it takes 4
 // consecutive elements, one 16-byte load per split.  Eight splits are summed pairwise before they are
@@ -2799,7 +2800,7 @@ __global__ void splitk_reduce(const float* __restrict__ ws, T* __restrict__ y, c
 }
 
 // Split-K reduction with the fused 2x2/2 max-pool: each pooled output sums the KS partial planes
-// at its four positions (split order), takes the maximum, adds the bias and applies ReLU.  The
+// at its four positions (pairwise, as above), takes the maximum, adds the bias and applies ReLU.  The
 // loads of 4 splits (16 loads) are issued before they are added.
 template <typename T>
 __global__ void splitk_reduce_pool(const float* __restrict__ ws, T* __restrict__ y, const float* __restrict__ bias,

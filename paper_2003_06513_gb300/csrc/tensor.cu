@@ -10,18 +10,26 @@
 // Precision.  Every fp32 operand is held as two fp16 values, v = (h + l 2^-11) 2^-k with one
 // power of two k per layer (weights) or per stage (inputs: 16 channels of the staged positions),
 // so the pair carries 22 to 23 bits down to 2^-28 of the largest value.  A chain of MMAs first sums
-// the cross terms h_x l_w + l_x h_w of three taps, then adds h_x h_w with the accumulator scaled
+// the cross terms h_x l_w + l_x h_w of the nine taps, then adds h_x h_w with the accumulator scaled
 // by 2^-11 in the first of those MMAs (scale-input-d); the dropped l_x l_w is 2^-24.6 of a product
-// (rms).  The tensor core's accumulator truncates, so a chain covers three taps of 16 channels
-// only and the sums are then added in fp32 registers, rounded to nearest, by eight warps.
-// fp16 inputs are exact, need two products and take chains of nine taps.
+// (rms), and tiles of one column block (MT 1: small batches, where the FFMA kernel's split sums round
+// less) sum it as well.  The tensor core's accumulator truncates, so a chain covers 16 channels
+// only and the sums are then added in fp32 registers, rounded to nearest, by eight warps; what the
+// truncation takes away on average is put back into the weights (wbias below).
+// fp16 inputs are exact and need two products.
+//
+// Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 198,
+// 512->512 14x14 183 -> 70, 64->64 224x224 with the pool 547 -> 351, 128->128 56x56 stride 2
+// 200 -> 54; fp16 256->256 28x28 keep 1 808 -> 73.  What bounds it: 12 % over the bare MMA stream
+// (175 us) on the 56x56 and 28x28 layers of 256 and 512 filters, the input staging (six warps:
+// load, split into pairs, store) with 64 filters or stride 2, one partial wave of CTA pairs on the
+// smallest.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <atomic>
 #include <climits>
-#include <cstdlib>
 #include <cstdint>
 
 #include "tensor.h"
