@@ -251,9 +251,10 @@ int pp_conv_plan_dt(pp_handle h, int dtype, int pool, int N, int H, int W, size_
  * info[0] = 1 if so (else 0 and zeros), [1] input-channel splits, [2] workspace bytes used, [3] work
  * units (pairs of position tiles x filter chunks x splits), [4] positions of a tile, [5] filters of a
  * unit, [6] and [7] width and height of a tile that is a rectangle of outputs (0: consecutive
- * positions of the whole batch).  Calls that do not take it run the plan of pp_conv_plan_dt, as all
+ * positions of the whole batch), [8] 1 where 16-byte aligned input comes by tensor copies of whole
+ * windows.  Calls that do not take it run the plan of pp_conv_plan_dt, as all
  * calls of a layer without pp_bind_tensor do; the workspace to pass is that plan's in either case.
- * Writes min(n_info, 8) values.  Errors as pp_conv_plan_dt.  Host-only. */
+ * Writes min(n_info, 9) values.  Errors as pp_conv_plan_dt.  Host-only. */
 int pp_conv_tensor_plan(pp_handle h, int dtype, int pool, int N, int H, int W, size_t workspace_bytes,
                         int64_t* info, int n_info);
 

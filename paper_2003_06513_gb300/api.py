@@ -147,7 +147,7 @@ class Layer:
         return d
 
     TENSOR_PLAN_KEYS = ("tensor", "splits", "workspace_bytes", "units", "positions", "filters",
-                        "tile_w", "tile_h")
+                        "tile_w", "tile_h", "boxes")
 
     def tensor_plan(self, x_shape, workspace_bytes: int = 0, pool2x2: bool = False,
                     dtype=torch.float32) -> dict:

@@ -3494,6 +3494,16 @@ bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
 
 }  // namespace
 
+bool patconv::encode_box(CUtensorMap* map, const void* x, int N, int C, int H, int W, int rw, int rows) {
+    if (!encode_tiled()) return false;
+    const cuuint64_t dims[4] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)C, (cuuint64_t)N};
+    const cuuint64_t strides[3] = {(cuuint64_t)W * 4, (cuuint64_t)H * W * 4, (cuuint64_t)C * H * W * 4};
+    const cuuint32_t box[4] = {(cuuint32_t)rw, (cuuint32_t)rows, 16, 1}, estr[4] = {1, 1, 1, 1};
+    return encode_tiled()(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(x), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 extern "C" {
 
 int pp_bind_device(pp_handle h, void* dev_image, size_t bytes, void* stream) {
@@ -3680,7 +3690,7 @@ int pp_conv_tensor_plan(pp_handle h, int dtype, int pool, int N, int H, int W, s
     if (pool != 0 && pool != 1) return PP_ERR_ARG;
     if (pool && (h->depthwise || !h->fast)) return PP_ERR_PATH;
     if (N < 1 || H < 1 || W < 1 || n_info < 1) return PP_ERR_SHAPE;
-    int64_t v[8] = {0};
+    int64_t v[9] = {0};
     Plan pl;
     const size_t ws = h->fast ? workspace_bytes : 0;
     if (!h->depthwise && make_plan(h, N, H, W, ws, &pl, pool, true, dtype == PP_F32 ? 4 : 2) == PP_OK && pl.tensor) {
@@ -3692,8 +3702,9 @@ int pp_conv_tensor_plan(pp_handle h, int dtype, int pool, int N, int H, int W, s
         v[5] = pl.tc.NC;
         v[6] = pl.tc.tw;
         v[7] = pl.tc.th;
+        v[8] = pl.tc.box;
     }
-    for (int i = 0; i < n_info && i < 8; ++i) info[i] = v[i];
+    for (int i = 0; i < n_info && i < 9; ++i) info[i] = v[i];
     return PP_OK;
 }
 

@@ -24,6 +24,7 @@
 // (175 us) on the 56x56 and 28x28 layers of 256 and 512 filters, the input staging (six warps:
 // load, split into pairs, store) with 64 filters or stride 2, one partial wave of CTA pairs on the
 // smallest.
+#include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -31,6 +32,7 @@
 #include <atomic>
 #include <climits>
 #include <cstdint>
+#include <cstring>
 
 #include "tensor.h"
 
@@ -42,7 +44,7 @@ constexpr int kPromoteWarps = 8;        // warps 0-7: sums in registers, epilogu
 constexpr int kProducerWarps = 6;       // warps 8-13: input staging
 constexpr int kLoaderWarp = 14, kMmaWarp = 15;
 constexpr int kProducers = kProducerWarps * 32;
-constexpr int kMaxWSlots = 12, kMaxXStages = 4;
+constexpr int kMaxWSlots = 12, kMaxXStages = 4, kMaxRaw = 3;
 // items a producer thread's copies run ahead, plus one, by the words of a channel in an item
 constexpr int ring_of(int words) { return words == 1 ? 6 : (words == 2 ? 4 : 3); }
 constexpr int kHdr = 8;                 // stage headers in flight
@@ -89,6 +91,7 @@ struct TcParams {
     int tiles, n_fchunks, n_units;
     int vec, ppr, n_entries, items;   // values a copy; copies of a staged row (vec > 1); table entries; items of a block
     FastDiv d_ip, d_wp, d_p, d_ppr;
+    int box, rw, rs;           // input by boxes of rows of rw values; their stages
     float* ws;
     size_t ws_stride;
     int xs, hs, ls;            // input stages, slots of the hi and lo weights
@@ -194,6 +197,11 @@ __device__ __forceinline__ bool wait_bar(uint32_t a, uint32_t parity, const TcPa
 __device__ __forceinline__ bool wait_warp(uint32_t a, uint32_t parity, const TcParams& p, volatile int* abort_flag,
                                           unsigned code) {
     return __all_sync(0xFFFFFFFFu, wait_bar(a, parity, p, abort_flag, code));
+}
+__device__ __forceinline__ void box_load(uint32_t dst, const CUtensorMap* map, int x, int y, int c, int n, uint32_t mbar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(c), "r"(n), "r"(mbar) : "memory");
 }
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -685,6 +693,132 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
     }
 }
 
+// Staging from boxes (stride 1, fp32, rectangles, rows of a multiple of 16 bytes): one tensor copy
+// brings a block's window, 16 channels of th + 2 rows from the 16-byte boundary left of it, with zeros
+// outside the image and beyond the last channel; the six warps only read, split and store, neighbouring
+// lanes neighbouring positions.  With produce_async, a third of these warps' time went into issuing
+// copies (some 1300 clocks for eight by each warp, all six at once after the block's barrier, the
+// copies' data long there when it was wanted).  64 -> 64 at 224x224 with the pool, batch 32:
+// 351 -> 320 us, 64 -> 128 at 112x112 153 -> 135; the next item's values are read before this one is
+// split (323 without that, 370 with four items unrolled).
+__device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap* map, unsigned char* smem, uint32_t xfull, uint32_t xempty,
+                                            uint32_t rfull, volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
+    const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
+    const int cw = (p.th + 2) * p.rw;                // words of a channel's box
+    const uint32_t bytes = 64u * (uint32_t)cw;       // of a box: a multiple of 256
+    // the copies' cursor (thread 0): unit, block
+    int iu = pair, icb = 0, icb1 = 0, issued = 0, x0 = 0, y0 = 0, n0 = 0;
+    auto issue = [&]() {
+        if (iu >= p.n_units) return;
+        if (icb == icb1) {
+            const Unit U = unit_of(p, iu, rank);
+            icb = U.cb0;
+            icb1 = U.cb1;
+            x0 = (U.ox0 - 1) & ~3;                   // 16-byte boundary
+            y0 = U.oy0 - 1;
+            n0 = U.n;
+        }
+        const uint32_t s = (uint32_t)(issued % p.rs), bar = rfull + 8 * s;
+        mbar_expect_tx(bar, bytes);
+        box_load(smem_u32(smem) + p.ring_off + s * bytes, map, x0, y0, 16 * icb, n0, bar);
+        ++issued;
+        if (++icb == icb1) iu += pairs;
+    };
+    int done = 0, slot = 0, ph = 0;                  // blocks taken, their stage, its use
+    // nothing in flight at the exit: after a timeout the boxes asked for land first
+    auto drain = [&]() {
+        if (tid != 0 || done == issued) return;
+        const long long t0 = clock64();
+        for (; done < issued; ++done)
+            while (!mbar_try(rfull + 8 * (done % p.rs), (uint32_t)(done / p.rs) & 1u) && clock64() - t0 < kDrainCycles) {}
+        if (clock64() - t0 >= kDrainCycles) atomicOr(p.status, kErrDrain);
+    };
+    if (tid == 0)
+        for (int r = 0; r < p.rs; ++r) issue();
+    int kexp = 0;
+    Stage sg;
+    for (int u = pair; u < p.n_units; u += pairs) {
+        const Unit U = unit_of(p, u, rank);
+        const int shift = (U.ox0 - 1) & 3, blocks = U.cb1 - U.cb0;
+        for (int cb = 0; cb < blocks; ++cb) {
+            bool ok = sg.e < p.xs || wait_bar(xempty + 8 * sg.s, (sg.ph & 1) ^ 1, p, abort_flag, kErrSpace);
+            ok = ok && wait_bar(rfull + 8 * slot, (uint32_t)ph & 1u, p, abort_flag, kErrData);
+            unsigned char* st = smem + p.x_off + (size_t)sg.s * p.x_stage;
+            const float* raw = reinterpret_cast<const float*>(smem + p.ring_off + (uint32_t)slot * bytes) + shift;
+            uint32_t mn = 0xFFFFFFFFu, mx = 0;
+            __half2 hmx = __half2half2(__ushort_as_half(0));
+            float scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
+            // item i: eight channels of a staged position (zeros: the two positions after the last row)
+            auto take = [&](int i, float (&v)[8]) {
+                const int k = i >= p.P ? 1 : 0, q = i - k * p.P, r = (int)fdiv((uint32_t)q, p.d_wp);
+                const float* f = raw + 8 * k * cw + r * p.rw + (q - r * p.Wp);
+                const bool in = r < p.th + 2;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = in ? f[j * cw] : 0.0f;
+                return st + (uint32_t)k * p.plane + 16u * (uint32_t)q;
+            };
+            auto put = [&](const float (&v)[8], unsigned char* d) {
+                // the smallest |v| as an ordered integer, a zero as the largest
+#pragma unroll
+                for (int j = 0; j < 8; j += 2)
+                    mn = min(min(mn, 2u * __float_as_uint(v[j]) - 1u), 2u * __float_as_uint(v[j + 1]) - 1u);
+                uint4 hi, lo;
+                split8(v, scale, &hi, &lo, &hmx);
+                *reinterpret_cast<uint4*>(d) = hi;
+                *reinterpret_cast<uint4*>(d + 2 * p.plane) = lo;
+            };
+            if (ok) {
+                float v[8];
+                unsigned char* d = take(tid, v);
+                for (int i = tid; i < 2 * p.P; i += kProducers) {
+                    float w[8];
+                    unsigned char* dn = d;
+                    if (i + kProducers < 2 * p.P) dn = take(i + kProducers, w);
+                    put(v, d);
+                    d = dn;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = w[j];
+                }
+            }
+            // the larger half of the largest hi parts; NaN is the largest of all
+            const uint32_t b = *reinterpret_cast<const uint32_t*>(&hmx);
+            mx = max(b & 0xFFFFu, b >> 16);
+            if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return drain();
+            // as in produce_async: a block beyond the scale is taken again
+            int ex = (int)(mx >> 10) - 15 - kexp;
+            bool slow = false;
+            if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
+                mx = 0;
+#pragma unroll 1
+                for (int i = tid; i < 2 * p.P; i += kProducers) {
+                    float v[8];
+                    take(i, v);
+                    for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[j]));
+                }
+                if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return drain();
+                ex = (int)(mx >> 24) - 127;
+                slow = ex < -60 || ex > 120;   // also infinities and NaN
+                if (!slow) {
+                    kexp = 13 - ex;
+                    scale = __uint_as_float((uint32_t)(127 + kexp) << 23);
+#pragma unroll 1
+                    for (int i = tid; i < 2 * p.P; i += kProducers) {
+                        float v[8];
+                        unsigned char* d = take(i, v);
+                        put(v, d);
+                    }
+                    bar_or<1, kProducers>(false);   // all have read the box
+                }
+            }
+            slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
+            ++done;
+            if (++slot == p.rs) { slot = 0; ++ph; }
+            if (tid == 0) issue();                  // into the stage just read
+            publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
+        }
+    }
+}
+
 // fp16 rows of odd length, or inputs aligned to one value only: loads run two items ahead in registers.
 template <int S>
 __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
@@ -852,7 +986,7 @@ __device__ __noinline__ void general_unit(const TcParams& p, const Unit& U, int 
 // ---------------------------------------------------------------------------- the kernel
 
 template <int S, typename T, int MT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_tc(const __grid_constant__ TcParams p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_tc(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
     constexpr int M = 128 * MT;
     constexpr int HL = sizeof(T) == 4 ? 2 : 1;
     constexpr int TCOL = 256 / MT;                // accumulator columns of a 128-position tile
@@ -863,7 +997,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     const uint32_t bar0 = smem_u32(smem);
     const uint32_t xfull = bar0, xempty = xfull + 8 * kMaxXStages, hfull = xempty + 8 * kMaxXStages,
                    hempty = hfull + 8 * kMaxWSlots, lfull = hempty + 8 * kMaxWSlots, lempty = lfull + 8 * kMaxWSlots,
-                   tfull = lempty + 8 * kMaxWSlots, tempty = tfull + 16, drain = tempty + 16;
+                   tfull = lempty + 8 * kMaxWSlots, tempty = tfull + 16, drain = tempty + 16, rfull = drain + 8;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + 640);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 644);
     float2* hdr = reinterpret_cast<float2*>(smem + 704);
@@ -890,6 +1024,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 mbar_init(tempty + 8 * i, 2 * kPromoteWarps);
             }
             mbar_init(drain, 1);
+            for (int i = 0; i < kMaxRaw; ++i) mbar_init(rfull + 8 * i, 1);
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
@@ -1050,7 +1185,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
-            if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            if (S == 1 && HL == 2 && p.box) produce_box(p, &tmap, smem, xfull, xempty, rfull, abort_flag, red, hdr, rank, pair, pairs);
+            else if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else if (p.vec == 2) produce_async<S, T, 2>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else if constexpr (HL == 2) produce_async<S, T, 1>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
@@ -1292,7 +1428,7 @@ void fill_layer(const pp_layer* L, TcParams* p) {
     for (int i = 0; i < kMaxPatterns; ++i) p->masks[i] = L->masks[i];
 }
 
-using TcKernel = void (*)(const TcParams);
+using TcKernel = void (*)(const TcParams, const CUtensorMap);
 
 template <int S, typename T, int MT>
 TcKernel pick(size_t need) {
@@ -1398,7 +1534,10 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         const double mma = 9.0 * (HL + 1 + ll) * c.MT * std::max(c.NC / 2.0, 32.0 + c.NC / 8.0) + 200.0;
         // a copy brings one, two or four values, where rows are a multiple of them (and x is aligned:
         // tensor_launch)
-        for (int vec = 1; vec <= 4 && W % vec == 0; vec *= 2) {
+        for (int way = 1; way <= 8 && W % std::min(way, 4) == 0; way *= 2) {
+            const int vec = std::min(way, 4);
+            c.box = way == 8;
+            if (c.box && (es != 4 || S != 1 || !c.tw)) continue;
             c.vec = vec;
             const int np = std::max(1, vec / S);   // positions of a copy
             c.ppr = c.tw ? (c.Wp + 2 * (np - 1)) / np : Wo / np + 1;
@@ -1411,6 +1550,13 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             c.ring_off = (unsigned)align_up(c.tab_off + std::max<size_t>(4 * (size_t)c.P, 8 * (size_t)c.n_entries), 128);
             const int words = es == 4 ? vec : std::max(1, vec / 2);
             c.x_off = c.ring_off + std::max(ring_of(1) * 9, ring_of(words) * (8 * words + 1)) * kProducers * 4;
+            if (c.box) {   // two or three boxes; the copies' ring, should x not be aligned, in their place
+                c.rw = (3 + c.Wp + 3) & ~3;
+                const size_t box = (size_t)64 * (c.th + 2) * c.rw;
+                if (c.rw > 256 || c.th + 2 > 256) continue;
+                c.rs = 2;
+                c.x_off = (unsigned)(c.ring_off + std::max(align_up(c.rs * box, 128), (size_t)ring_of(1) * 9 * kProducers * 4));
+            }
             if (c.x_off >= kSmemMax) continue;
             const size_t left = kSmemMax - c.x_off;
             // three input stages with two blocks' weights, else two with at least a block's and a row
@@ -1434,7 +1580,8 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             // towards the fast ones; the choice is 1.5 % from the best on average).
             static const double kRound[2][3] = {{840.0, 1280.0, 1920.0}, {840.0, 945.0, 1030.0}};   // fp32, fp16
             const int rounds = (c.items + kProducers - 1) / kProducers;
-            const double staging = rounds * kRound[es == 2][vec == 1 ? 0 : vec / 2];
+            // boxes: 400 clocks a round of eight channels (250 took layers that ran 1 % slower so)
+            const double staging = c.box ? (2.0 * c.P + kProducers - 1) / kProducers * 400.0 : rounds * kRound[es == 2][vec == 1 ? 0 : vec / 2];
             const double stage = (mma + std::max(0.0, staging - 0.64 * mma)) * (c.hs + c.ls < 8 ? 1.09 : 1.0);
             for (int ks = 1; ks <= c.n_cb && (ks == 1 || units1 * ks <= 2 * pairs); ++ks) {
                 const int cbs = (c.n_cb + ks - 1) / ks;
@@ -1515,7 +1662,12 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.x_off = pl.x_off;
     p.h_off = pl.h_off;
     p.l_off = pl.l_off;
-    if (pl.vec > 1 && reinterpret_cast<uintptr_t>(c.x) % (pl.vec * (size_t)c.es) != 0) {   // single pixels after all
+    p.rw = pl.rw;
+    p.rs = pl.rs;
+    CUtensorMap tmap;
+    std::memset(&tmap, 0, sizeof(tmap));
+    p.box = pl.box && reinterpret_cast<uintptr_t>(c.x) % 16 == 0 && encode_box(&tmap, c.x, c.N, p.C, c.H, c.W, pl.rw, pl.th + 2);
+    if (pl.box ? !p.box : pl.vec > 1 && reinterpret_cast<uintptr_t>(c.x) % (pl.vec * (size_t)c.es) != 0) {   // single pixels after all
         p.vec = 1;
         p.n_entries = pl.P;
         p.items = 2 * pl.P * (L->stride == 1 ? 1 : 4);
@@ -1535,7 +1687,7 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     cfg.stream = c.st;
     cfg.attrs = attr;
     cfg.numAttrs = c.pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, p, tmap);
     const cudaError_t l = cudaGetLastError();
     return e != cudaSuccess ? e : l;
 }

@@ -3,6 +3,10 @@
 
 #include <cstddef>
 
+#ifdef __CUDACC__
+#include <cuda.h>
+#endif
+
 #include "layer.h"
 
 namespace patconv {
@@ -19,6 +23,7 @@ struct TensorPlan {
     int mstep = 0;          // flat tiles: positions a tile advances
     int P = 0;              // positions a tile stages
     int vec = 1, ppr = 0, n_entries = 0, items = 0;   // values a copy, copies of a staged row, table, items
+    int box = 0, rw = 0, rs = 0;   // input by tensor copies of 16 channels: values of a row, stages
     int tw = 0, th = 0, tiles_x = 0, tiles_y = 0;   // rectangles of outputs (tw 0: flat tiles)
     int tiles = 0, n_fchunks = 0;   // tiles: pairs of position tiles, one per CTA of a pair
     long long units = 0;
@@ -51,6 +56,8 @@ struct TensorCall {
 bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_t ws_bytes, int sms, TensorPlan* out,
                  int ll = 0);
 #ifdef __CUDACC__
+// Tensor map of fp32 x [N][C][H][W] with boxes of 16 channels of `rows` rows of `rw` values (conv.cu).
+bool encode_box(CUtensorMap* map, const void* x, int N, int C, int H, int W, int rw, int rows);
 cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl);
 // Builds the tensor-core weights from the bound device image.
 cudaError_t tensor_build_weights(const pp_layer* L, void* dst, cudaStream_t st);

@@ -237,3 +237,28 @@ def test_bind_tensor_errors():
     assert lib.pp_bind_tensor(api.pp_pack(W, None, 0.5)._h, p(), n, None) == -8
     dw = api.pp_pack(W[:, :1], None, 1.0, 32).bind("cuda")
     assert dw.query("tensor_bytes") == 0 and lib.pp_bind_tensor(dw._h, p(), n, None) == -14
+
+
+@pytest.mark.parametrize("case", [(64, 72, 5, 60, 100, False), (64, 64, 3, 57, 148, False), (128, 72, 7, 50, 112, False),
+                                  (128, 40, 5, 80, 112, True), (64, 72, 9, 61, 100, True), (64, 72, 33, 33, 100, True)])
+def test_tensor_kernel_takes_its_input_by_boxes(case):
+    """Tensor copies of whole windows: tiles narrower than the rows and not, all shifts to the 16-byte
+    boundary, a last block of 8 channels, an odd number of tiles; channels of other ranges make blocks
+    be taken again.  x one element off the boundary takes single copies: the same values staged, so the
+    same result, bit for bit.  An infinity reaches the outputs that it reaches on the CUDA cores."""
+    cout, cin, n, h, w, pool = case
+    layer, W, b = _layer(cout, cin, 0.5, 1, cin + w)
+    x = WL.activations((n, cin, h, w), 7 + h, relu=True, dtype=np.float32)
+    x[:, 16:32] *= np.float32(2.0 ** 14)
+    x[n // 2, :16] *= np.float32(2.0 ** -12)
+    bt = torch.from_numpy(b).cuda()
+    xt = torch.from_numpy(x).cuda()
+    assert layer.tensor_plan(xt.shape, 0, pool)["boxes"] == 1
+    y = layer.conv(xt, bt, True, pool2x2=pool)
+    _check(y, x, W, b, 0.5, 1, pool, "f32", idx=[0, n // 2, n - 1])
+    off = torch.empty(xt.numel() + 1, device="cuda")[1:].view(xt.shape).copy_(xt)
+    assert torch.equal(layer.conv(off, bt, True, pool2x2=pool), y)
+    xt[n - 1, cin - 1, h - 1, w - 2] = float("inf")
+    y = layer.conv(xt, bt, False, pool2x2=pool)
+    ref = _cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
+    assert torch.equal(torch.isfinite(y), torch.isfinite(ref)) and not torch.isfinite(y).all()
