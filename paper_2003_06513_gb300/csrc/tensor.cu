@@ -19,10 +19,10 @@
 // fp16 inputs are exact and need two products.
 //
 // Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 198,
-// 512->512 14x14 183 -> 70, 64->64 224x224 with the pool 547 -> 351, 128->128 56x56 stride 2
+// 512->512 14x14 183 -> 70, 64->64 224x224 with the pool 547 -> 326, 256->256 28x28 stride 2
 // 200 -> 54; fp16 256->256 28x28 keep 1 808 -> 73.  What bounds it: 12 % over the bare MMA stream
 // (175 us) on the 56x56 and 28x28 layers of 256 and 512 filters, the input staging (six warps:
-// load, split into pairs, store) with 64 filters or stride 2, one partial wave of CTA pairs on the
+// split into pairs, store) with 64 filters or stride 2, one partial wave of CTA pairs on the
 // smallest.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -651,12 +651,16 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                 // (from memory), its largest value scaled to [2^13, 2^14)
                 int ex = (int)(mx >> 10) - 15 - kexp;
                 if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
-                    const int n0 = first_image(p, U);
+                    int u1 = u;
+                    asm volatile("" : "+r"(u1));   // the unit again: held in registers for this rare path it cost
+                                                   // spills (28x28 stride 2, batch 64: 55.7 -> 53.6 us)
+                    const Unit U1 = unit_of(p, u1, rank);
+                    const int n0 = first_image(p, U1);
                     auto again = [&](int i, float (&v)[V][8]) {
                         uint32_t off, dst;
                         const bool in = decode(i, [&](int m) {
-                            if constexpr (VEC > 1) return copy_entry<S, VEC>(p, U, m, n0);
-                            else return make_uint2(window_entry<S>(p, U, m, n0), 0u);
+                            if constexpr (VEC > 1) return copy_entry<S, VEC>(p, U1, m, n0);
+                            else return make_uint2(window_entry<S>(p, U1, m, n0), 0u);
                         }, &off, &dst);
                         const int nch = in ? p.C - cb * 16 - channel_of(i) : 0;
                         const float* src = static_cast<const float*>(p.x) + ((size_t)n0 * p.C + cb * 16) * HW + off;
@@ -699,8 +703,8 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
 // lanes neighbouring positions.  With produce_async, a third of these warps' time went into issuing
 // copies (some 1300 clocks for eight by each warp, all six at once after the block's barrier, the
 // copies' data long there when it was wanted).  64 -> 64 at 224x224 with the pool, batch 32:
-// 351 -> 320 us, 64 -> 128 at 112x112 153 -> 135; the next item's values are read before this one is
-// split (323 without that, 370 with four items unrolled).
+// 351 -> 326 us, 64 -> 128 at 112x112 153 -> 135; the next item's values are read before this one is
+// split (334 against 328 in the benchmark's step; 375 with four items unrolled).
 __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap* map, unsigned char* smem, uint32_t xfull, uint32_t xempty,
                                             uint32_t rfull, volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
     const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
