@@ -1189,7 +1189,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
-            if (S == 1 && HL == 2 && p.box) produce_box(p, &tmap, smem, xfull, xempty, rfull, abort_flag, red, hdr, rank, pair, pairs);
+            if (S == 1 && HL == 2 && MT > 1 && p.box) produce_box(p, &tmap, smem, xfull, xempty, rfull, abort_flag, red, hdr, rank, pair, pairs);
             else if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else if (p.vec == 2) produce_async<S, T, 2>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
             else if constexpr (HL == 2) produce_async<S, T, 1>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
@@ -1541,7 +1541,9 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
         for (int way = 1; way <= 8 && W % std::min(way, 4) == 0; way *= 2) {
             const int vec = std::min(way, 4);
             c.box = way == 8;
-            if (c.box && (es != 4 || S != 1 || !c.tw)) continue;
+            // (not for tiles of 128: with this path in it their kernel ran 1 % slower on flat tiles,
+            // 256 -> 256 at 56x56 201.6 against 199.9 us)
+            if (c.box && (es != 4 || S != 1 || !c.tw || c.MT == 1)) continue;
             c.vec = vec;
             const int np = std::max(1, vec / S);   // positions of a copy
             c.ppr = c.tw ? (c.Wp + 2 * (np - 1)) / np : Wo / np + 1;
