@@ -51,6 +51,7 @@ constexpr int kHdr = 8;                 // stage headers in flight
 constexpr unsigned kHeadBytes = 1024 + 2 * 256 * 4;   // barriers, headers, two units' biases
 constexpr uint32_t kTmemColumns = 512;
 constexpr long long kDrainCycles = 2000000000LL;   // about one second
+constexpr long long kSettleCycles = 20000;         // about 10 us
 constexpr unsigned kErrData = 1u, kErrSpace = 2u, kErrDrain = 4u;
 
 // division of 0 <= n < 2^31 by a constant d >= 2
@@ -378,6 +379,16 @@ __device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t x
     if (++sg->s == p.xs) { sg->s = 0; ++sg->ph; }
 }
 
+// The end of staging: the MMAs' last commits signal xempty in both CTAs of the pair, also for stages
+// that nobody fills again, and a CTA must not exit before these arrivals have landed in its shared
+// memory.  One thread waits for the last use of every stage (the uses before it were waited for when
+// the stage was filled again).
+__device__ __forceinline__ void stages_done(const TcParams& p, const Stage& sg, uint32_t xempty, volatile int* abort_flag, int tid) {
+    if (tid != 0) return;
+    for (int k = max(0, sg.e - p.xs); k < sg.e; ++k)
+        if (!wait_bar(xempty + 8 * (k % p.xs), (uint32_t)(k / p.xs) & 1u, p, abort_flag, kErrSpace)) return;
+}
+
 // Item i of a block: plane and channel half k, position.
 template <int S>
 __device__ __forceinline__ bool item_of(const TcParams& p, int i, int items, int* k, int* pos) {
@@ -695,6 +706,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
             publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
         }
     }
+    stages_done(p, sg, xempty, abort_flag, tid);
 }
 
 // Staging from boxes (stride 1, fp32, rectangles, rows of a multiple of 16 bytes): one tensor copy
@@ -821,6 +833,7 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
             publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
         }
     }
+    stages_done(p, sg, xempty, abort_flag, tid);
 }
 
 // fp16 rows of odd length, or inputs aligned to one value only: loads run two items ahead in registers.
@@ -912,6 +925,7 @@ __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* sm
             if (cb >= U.cb1) break;
         }
     }
+    stages_done(p, sg, xempty, abort_flag, tid);
 }
 
 // ---------------------------------------------------------------------------- general sums
@@ -1225,9 +1239,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                     src += k % 3 == 2 ? 4 * p.w_slot : p.w_slot;
                 }
             }
-            // nothing of this CTA in flight at its exit: the slots filled last have landed
-            const long long t0 = clock64();
+            // nothing of this CTA in flight at its exit: the slots filled last have landed, and so have
+            // the arrivals of the commits that free them (as in stages_done)
             const int nl = lph * p.ls + lsl, nh = hph * p.hs + hsl;
+            for (int k = max(0, nl - p.ls); k < nl && ok; ++k)
+                ok = wait_warp(lempty + 8 * (k % p.ls), (uint32_t)(k / p.ls) & 1u, p, abort_flag, kErrSpace);
+            for (int k = max(0, nh - p.hs); k < nh && ok; ++k)
+                ok = wait_warp(hempty + 8 * (k % p.hs), (uint32_t)(k / p.hs) & 1u, p, abort_flag, kErrSpace);
+            const long long t0 = clock64();
             for (int k = max(0, nl - p.ls); k < nl; ++k)
                 while (!mbar_try(lfull + 8 * (k % p.ls), (uint32_t)(k / p.ls) & 1u) && clock64() - t0 < kDrainCycles) {}
             for (int k = max(0, nh - p.hs); k < nh; ++k)
@@ -1365,6 +1384,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 const long long t0 = clock64();
                 while (!mbar_try(drain, 0))
                     if (clock64() - t0 > kDrainCycles) { atomicOr(p.status, kErrDrain); break; }
+                // arrivals of the commits before it may still be on their way to the peer: they get 10 us
+                for (const long long t1 = clock64(); clock64() - t1 < kSettleCycles;) {}
             }
         }
     }

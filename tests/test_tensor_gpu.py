@@ -262,3 +262,23 @@ def test_tensor_kernel_takes_its_input_by_boxes(case):
     y = layer.conv(xt, bt, False, pool2x2=pool)
     ref = _cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
     assert torch.equal(torch.isfinite(y), torch.isfinite(ref)) and not torch.isfinite(y).all()
+
+
+@pytest.mark.parametrize("dtype,cin,h,tile_w,boxes", [(torch.float16, 16, 28, 0, 0), (torch.float16, 16, 30, 30, 0),
+                                                      (torch.float32, 32, 28, 28, 1), (torch.float32, 32, 30, 30, 0)])
+def test_units_of_one_or_two_blocks_back_to_back(dtype, cin, h, tile_w, boxes):
+    """The shortest units and epilogues (16 filters, one or two 16-channel blocks), one unit a CTA pair:
+    a pair ends while the arrivals of its last commits are still under way, and the next launch takes
+    over its shared memory at once.  Every launch gives the same bits."""
+    layer, W, b = _layer(16, cin, 1.0, 1, 21)
+    x = WL.activations((64, cin, h, h), 22, relu=True, dtype=NP["f32" if dtype == torch.float32 else "f16"])
+    xt = torch.from_numpy(x).cuda()
+    plan = layer.tensor_plan(xt.shape, 0, False, dtype)
+    assert (plan["tensor"], plan["tile_w"], plan["boxes"]) == (1, tile_w, boxes) and plan["units"] <= 76
+    bt = torch.from_numpy(b).cuda()
+    first = layer.conv(xt, bt, True)
+    _check(first, x, W, b, 1.0, 1, False, "f32" if dtype == torch.float32 else "f16", idx=[0, 63])
+    outs = [torch.empty_like(first) for _ in range(4)]
+    for i in range(200):
+        layer.conv(xt, bt, True, out=outs[i % 4])
+    assert all(torch.equal(o, first) for o in outs)
