@@ -160,8 +160,12 @@ __device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t tx) {
     asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(tx) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t a) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
+}
 // Arrival on the leader's barrier at the same offset, with the CTA's scope: what it announces is
-// read by the tensor core only, after a proxy fence, or not at all.  (A cluster-wide release waits
+// read by the tensor core only, after a proxy fence, or not at all (a block's header goes from the
+// staging warps to the summing warps of its own CTA over a barrier of its own).  (A cluster-wide release waits
 // for the thread's loads in flight: the 56x56 layer 241 against 203 us; cluster-wide acquires cost a
 // wait some 200 clocks.)
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t a) {
@@ -368,10 +372,12 @@ __device__ __forceinline__ bool combine(uint32_t* mx, uint32_t* mn, bool ok, uin
     *par ^= 1;
     return true;
 }
-__device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t xfull, float2* hdr, int kexp, bool slow, int tid,
-                                        int lane) {
-    if (tid == 0)
+__device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t xfull, float2* hdr, uint32_t hready, int kexp, bool slow,
+                                        int tid, int lane) {
+    if (tid == 0) {   // (the slot's header of kHdr blocks ago was read before this block's stage was freed)
         hdr[sg->e & (kHdr - 1)] = make_float2(__uint_as_float((uint32_t)(127 - kexp - p.wexp) << 23), slow ? 1.0f : 0.0f);
+        mbar_arrive(hready + 8 * (sg->e & (kHdr - 1)));
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (lane == 0 && !p.no_fill) mbar_arrive_leader(xfull + 8 * sg->s);
@@ -488,7 +494,7 @@ __device__ __forceinline__ uint2 copy_entry(const TcParams& p, const Unit& U, in
 // 2-byte form, so VEC is 2 or 4.
 template <int S, typename T, int VEC>
 __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
-                                            volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
+                                            volatile int* abort_flag, uint2* red, float2* hdr, uint32_t hready, int rank, int pair, int pairs) {
     constexpr bool F32 = sizeof(T) == 4;
     static_assert(F32 || VEC > 1, "fp16 values are copied in pairs at least");
     constexpr int HL = F32 ? 2 : 1;
@@ -703,7 +709,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                 }
                 slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
             }
-            publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
+            publish(p, &sg, xfull, hdr, hready, kexp, slow, tid, lane);
         }
     }
     stages_done(p, sg, xempty, abort_flag, tid);
@@ -718,7 +724,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
 // 351 -> 326 us, 64 -> 128 at 112x112 153 -> 135; the next item's values are read before this one is
 // split (334 against 328 in the benchmark's step; 375 with four items unrolled).
 __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap* map, unsigned char* smem, uint32_t xfull, uint32_t xempty,
-                                            uint32_t rfull, volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
+                                            uint32_t rfull, volatile int* abort_flag, uint2* red, float2* hdr, uint32_t hready, int rank, int pair, int pairs) {
     const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
     const int cw = (p.th + 2) * p.rw;                // words of a channel's box
     const uint32_t bytes = 64u * (uint32_t)cw;       // of a box: a multiple of 256
@@ -830,7 +836,7 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
             ++done;
             if (++slot == p.rs) { slot = 0; ++ph; }
             if (tid == 0) issue();                  // into the stage just read
-            publish(p, &sg, xfull, hdr, kexp, slow, tid, lane);
+            publish(p, &sg, xfull, hdr, hready, kexp, slow, tid, lane);
         }
     }
     stages_done(p, sg, xempty, abort_flag, tid);
@@ -839,7 +845,7 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
 // fp16 rows of odd length, or inputs aligned to one value only: loads run two items ahead in registers.
 template <int S>
 __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* smem, uint32_t xfull, uint32_t xempty,
-                                            volatile int* abort_flag, uint2* red, float2* hdr, int rank, int pair, int pairs) {
+                                            volatile int* abort_flag, uint2* red, float2* hdr, uint32_t hready, int rank, int pair, int pairs) {
     constexpr int UN = 2;
     constexpr int NPL = S == 1 ? 1 : 4;
     const int tid = (int)threadIdx.x - kPromoteWarps * 32, lane = tid & 31, warp = tid >> 5;
@@ -909,7 +915,7 @@ __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* sm
                 uint32_t mn = 0;
                 failed = !combine<false>(&bad, &mn, ok, red, &sg.par, warp, lane);
                 if (failed) return;
-                publish(p, &sg, xfull, hdr, 0, bad != 0, tid, lane);
+                publish(p, &sg, xfull, hdr, hready, 0, bad != 0, tid, lane);
             }
             cb = ncb;
             g = ng;
@@ -1015,7 +1021,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     const uint32_t bar0 = smem_u32(smem);
     const uint32_t xfull = bar0, xempty = xfull + 8 * kMaxXStages, hfull = xempty + 8 * kMaxXStages,
                    hempty = hfull + 8 * kMaxWSlots, lfull = hempty + 8 * kMaxWSlots, lempty = lfull + 8 * kMaxWSlots,
-                   tfull = lempty + 8 * kMaxWSlots, tempty = tfull + 16, drain = tempty + 16, rfull = drain + 8;
+                   tfull = lempty + 8 * kMaxWSlots, tempty = tfull + 16, drain = tempty + 16, rfull = drain + 8, hready = rfull + 8 * kMaxRaw;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + 640);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 644);
     float2* hdr = reinterpret_cast<float2*>(smem + 704);
@@ -1043,6 +1049,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
             }
             mbar_init(drain, 1);
             for (int i = 0; i < kMaxRaw; ++i) mbar_init(rfull + 8 * i, 1);
+            for (int i = 0; i < kHdr; ++i) mbar_init(hready + 8 * i, 1);
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
@@ -1083,7 +1090,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
             for (int jb = 0; jb < 4; ++jb) act[jb] = ((128 * half + 32 * jb) % TCOL) < p.NC;
             for (int cb = U.cb0; cb < U.cb1 && ok; ++cb, ++e) {
                 const uint32_t b = e & 1u;
-                ok = wait_warp(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData);
+                ok = wait_warp(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData) &&
+                     wait_warp(hready + 8 * (e & (kHdr - 1)), (e / kHdr) & 1u, p, abort_flag, kErrData);
                 if (!ok) break;
                 fence_after();
                 const float2 h = hdr[e & (kHdr - 1)];
@@ -1203,11 +1211,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
-            if (S == 1 && HL == 2 && MT > 1 && p.box) produce_box(p, &tmap, smem, xfull, xempty, rfull, abort_flag, red, hdr, rank, pair, pairs);
-            else if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
-            else if (p.vec == 2) produce_async<S, T, 2>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
-            else if constexpr (HL == 2) produce_async<S, T, 1>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
-            else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, rank, pair, pairs);
+            if (S == 1 && HL == 2 && MT > 1 && p.box) produce_box(p, &tmap, smem, xfull, xempty, rfull, abort_flag, red, hdr, hready, rank, pair, pairs);
+            else if (p.vec == 4) produce_async<S, T, 4>(p, smem, xfull, xempty, abort_flag, red, hdr, hready, rank, pair, pairs);
+            else if (p.vec == 2) produce_async<S, T, 2>(p, smem, xfull, xempty, abort_flag, red, hdr, hready, rank, pair, pairs);
+            else if constexpr (HL == 2) produce_async<S, T, 1>(p, smem, xfull, xempty, abort_flag, red, hdr, hready, rank, pair, pairs);
+            else produce_f16<S>(p, smem, xfull, xempty, abort_flag, red, hdr, hready, rank, pair, pairs);
             asm volatile("cp.async.wait_all;" ::: "memory");   // after a timeout: nothing in flight at the exit
         } else if (warp == kLoaderWarp) {
             // ---- weights: a slot holds this CTA's half of the unit's filters for a row of three

@@ -282,3 +282,21 @@ def test_units_of_one_or_two_blocks_back_to_back(dtype, cin, h, tile_w, boxes):
     for i in range(200):
         layer.conv(xt, bt, True, out=outs[i % 4])
     assert all(torch.equal(o, first) for o in outs)
+
+
+@pytest.mark.parametrize("w,boxes", [(30, 0), (32, 1)])
+def test_both_ctas_of_a_pair_use_their_own_scales(w, boxes):
+    """Three tiles an image, so every second pair's tiles belong to two images, whose inputs are up to
+    2^40 apart: each CTA sums its blocks with the scales that its own staging warps published.  Each
+    image within the 2-norm bound of its own result; the same bits every time."""
+    layer, W, _ = _layer(64, 64, 0.5, 1, 23)
+    x = WL.activations((33, 64, 45, w), 24, relu=True)
+    s = 2.0 ** np.random.default_rng(25).integers(-20, 21, 33)
+    x = (x * s[:, None, None, None]).astype(np.float32)
+    xt = torch.from_numpy(x).cuda()
+    plan = layer.tensor_plan(xt.shape)
+    assert (plan["tensor"], plan["tile_w"], plan["tile_h"], plan["boxes"]) == (1, w, 15, boxes)
+    first = layer.conv(xt, None, True)
+    for i in (0, 1, 2, 15, 16, 31, 32):
+        _check(first, x, W, np.zeros(64, np.float32), 0.5, 1, False, "f32", idx=[i])
+    assert all(torch.equal(layer.conv(xt, None, True), first) for _ in range(50))
