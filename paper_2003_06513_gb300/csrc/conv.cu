@@ -2957,10 +2957,13 @@ int launch_tm(const pp_layer* L, const void* x, void* y, const float* bias, int 
     Plan pl;
     const int rc = make_plan(L, N, H, W, ws ? ws_bytes : 0, &pl, pool, true, (int)sizeof(T));
     if (rc != PP_OK) return rc;
-    if ((pl.KS > 1 || pl.streamk) && reinterpret_cast<uintptr_t>(ws) % 16 != 0) return PP_ERR_ALIGN;
+    const bool ws_aligned = reinterpret_cast<uintptr_t>(ws) % 16 == 0;
+    if ((pl.KS > 1 || pl.streamk) && !ws_aligned) return PP_ERR_ALIGN;
     // never planned: pool windows must lie in one block; blocks at 4j - 2 are fp32 only
     if ((pool && pl.shift == 1) || (pl.shift == 2 && sizeof(T) != 4)) return PP_ERR_SHAPE;
-    if (pl.tensor && L->tdev && tensor_enabled())
+    // (a tensor-core plan may split where the FFMA plan does not: a misaligned workspace, which the
+    // FFMA plan leaves alone, then leaves the call to it)
+    if (pl.tensor && L->tdev && tensor_enabled() && (pl.tc.KS == 1 || ws_aligned))
         return launch_tensor<T>(L, pl.tc, x, y, bias, relu, N, H, W, Ho, Wo, ws, st, pool);
     TmParams p{};
     p.x = x;

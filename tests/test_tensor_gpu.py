@@ -300,3 +300,19 @@ def test_both_ctas_of_a_pair_use_their_own_scales(w, boxes):
     for i in (0, 1, 2, 15, 16, 31, 32):
         _check(first, x, W, np.zeros(64, np.float32), 0.5, 1, False, "f32", idx=[i])
     assert all(torch.equal(layer.conv(xt, None, True), first) for _ in range(50))
+
+
+def test_misaligned_workspace_that_only_the_tensor_core_plan_would_split_into():
+    """The tensor-core plan splits here and the CUDA-core plan does not: a workspace off the 16-byte
+    boundary is left alone, as it always was, and the call runs on the CUDA cores."""
+    layer, W, b = _layer(24, 400, 1.0, 1, 26)
+    x = WL.activations((202, 400, 8, 4), 27, relu=True, dtype=np.float16)
+    xt, bt = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
+    ws = torch.full((1 << 22,), float("nan"), device="cuda")
+    nb = 4 * (ws.numel() - 1)
+    assert layer.tensor_plan(xt.shape, nb, False, xt.dtype)["splits"] > 1
+    assert layer.plan(xt.shape, nb, False, xt.dtype)["splits"] == 1
+    y = layer.conv(xt, bt, True, workspace=ws[1:])
+    assert torch.isnan(ws).all()
+    _check(y, x, W, b, 1.0, 1, False, "f16", idx=[0, 201])
+    assert torch.equal(y, _cuda_cores_only(layer).conv(xt, bt, True))
