@@ -374,13 +374,13 @@ __device__ __forceinline__ bool combine(uint32_t* mx, uint32_t* mn, bool ok, uin
 }
 __device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t xfull, float2* hdr, uint32_t hready, int kexp, bool slow,
                                         int tid, int lane) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0 && !p.no_fill) mbar_arrive_leader(xfull + 8 * sg->s);
     if (tid == 0) {   // (the slot's header of kHdr blocks ago was read before this block's stage was freed)
         hdr[sg->e & (kHdr - 1)] = make_float2(__uint_as_float((uint32_t)(127 - kexp - p.wexp) << 23), slow ? 1.0f : 0.0f);
         mbar_arrive(hready + 8 * (sg->e & (kHdr - 1)));
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncwarp();
-    if (lane == 0 && !p.no_fill) mbar_arrive_leader(xfull + 8 * sg->s);
     ++sg->e;
     if (++sg->s == p.xs) { sg->s = 0; ++sg->ph; }
 }
@@ -388,8 +388,9 @@ __device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t x
 // The end of staging: the MMAs' last commits signal xempty in both CTAs of the pair, also for stages
 // that nobody fills again, and a CTA must not exit before these arrivals have landed in its shared
 // memory.  One thread waits for the last use of every stage (the uses before it were waited for when
-// the stage was filled again).
-__device__ __forceinline__ void stages_done(const TcParams& p, const Stage& sg, uint32_t xempty, volatile int* abort_flag, int tid) {
+// the stage was filled again).  Not inlined: inside the staging loops' code it cost them registers
+// (64 bytes of spills more; 64 -> 64 at 224x224 with the pool 330 -> 337 us).
+__device__ __noinline__ void stages_done(const TcParams& p, const Stage& sg, uint32_t xempty, volatile int* abort_flag, int tid) {
     if (tid != 0) return;
     for (int k = max(0, sg.e - p.xs); k < sg.e; ++k)
         if (!wait_bar(xempty + 8 * (k % p.xs), (uint32_t)(k / p.xs) & 1u, p, abort_flag, kErrSpace)) return;
@@ -1090,8 +1091,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
             for (int jb = 0; jb < 4; ++jb) act[jb] = ((128 * half + 32 * jb) % TCOL) < p.NC;
             for (int cb = U.cb0; cb < U.cb1 && ok; ++cb, ++e) {
                 const uint32_t b = e & 1u;
-                ok = wait_warp(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData) &&
-                     wait_warp(hready + 8 * (e & (kHdr - 1)), (e / kHdr) & 1u, p, abort_flag, kErrData);
+                ok = wait_bar(hready + 8 * (e & (kHdr - 1)), (e / kHdr) & 1u, p, abort_flag, kErrData) &&
+                     wait_bar(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData);
+                ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 fence_after();
                 const float2 h = hdr[e & (kHdr - 1)];
