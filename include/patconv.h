@@ -145,7 +145,8 @@ int pp_bind_device(pp_handle h, void* dev_image, size_t bytes, void* stream);
  * fp16 values with a common power of two, zeros at the pruned taps; PP_Q_TENSOR_BYTES bytes) in
  * caller-owned DEVICE memory `dev` (256-byte aligned) from the device image bound before, enqueued
  * on `stream`.  The same rules as for the image: the caller keeps the memory alive and unmodified
- * while the handle is used and orders this call before the first pp_conv.  Later calls of pp_conv
+ * while the handle is used and orders this call before the first pp_conv.  The device of `dev` must
+ * be the current one (a kernel builds the weights).  Later calls of pp_conv
  * and its variants then take the tensor-core kernel wherever it is the faster one; results agree
  * to fp32 rounding.  Without this call they run on the CUDA cores.  pp_bind_device withdraws it.
  * Errors: PP_ERR_NULL, PP_ERR_NOT_BOUND, PP_ERR_PATH (PP_Q_TENSOR_BYTES is 0: depthwise layers and

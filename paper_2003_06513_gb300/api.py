@@ -102,20 +102,21 @@ class Layer:
         device = torch.device(device if device is not None else "cuda")
         if device.type != "cuda":
             raise ValueError("the packed image must live in CUDA device memory")
-        n = self.query("image_bytes")
-        buf = torch.empty(n, dtype=torch.uint8, device=device)
-        _lib.check("pp_bind_device", _lib.load().pp_bind_device(
-            self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
-        self._dev_buf = buf
-        self._tensor_buf = None
-        n = self.query("tensor_bytes")
-        if n:
+        with torch.cuda.device(device):     # pp_bind_tensor launches a kernel on the current device
+            n = self.query("image_bytes")
             buf = torch.empty(n, dtype=torch.uint8, device=device)
-            _lib.check("pp_bind_tensor", _lib.load().pp_bind_tensor(
+            _lib.check("pp_bind_device", _lib.load().pp_bind_device(
                 self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
-            self._tensor_buf = buf
-            if not torch.cuda.is_current_stream_capturing():
-                (stream if stream is not None else torch.cuda.current_stream(device)).synchronize()
+            self._dev_buf = buf
+            self._tensor_buf = None
+            n = self.query("tensor_bytes")
+            if n:
+                buf = torch.empty(n, dtype=torch.uint8, device=device)
+                _lib.check("pp_bind_tensor", _lib.load().pp_bind_tensor(
+                    self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
+                self._tensor_buf = buf
+                if not torch.cuda.is_current_stream_capturing():
+                    (stream if stream is not None else torch.cuda.current_stream(device)).synchronize()
         return self
 
     def out_shape(self, x_shape) -> tuple:
