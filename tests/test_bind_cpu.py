@@ -99,3 +99,14 @@ def test_the_layers_device_is_current_at_every_call(fake):
     _dense().bind("cuda:1")
     assert [c[:2] for c in fake.calls if c[0] != "done"] == [("image", 1), ("tensor", 1)]
     assert fake.current == 0
+
+
+def test_complete_on_return_whatever_the_layer_holds(fake):
+    """Depthwise layers and weights of extreme range have no tensor-core weights; their image is copied
+    all the same, and calls on any stream may follow."""
+    w = np.random.default_rng(0).standard_normal((16, 1, 3, 3)).astype(np.float32)
+    for layer, builds in ((_dense(), True), (api.pp_pack(w, None, 1.0, 16), False),
+                          (api.pp_pack(np.full((8, 16, 3, 3), 1e-20, np.float32), None, 1.0), False)):
+        fake.calls.clear()
+        layer.bind("cuda")
+        assert [c[0] for c in fake.calls] == ["image"] + ["tensor"] * builds + ["done"]
