@@ -115,8 +115,11 @@ class Layer:
                 _lib.check("pp_bind_tensor", _lib.load().pp_bind_tensor(
                     self._h, ctypes.c_void_p(buf.data_ptr()), n, _stream_ptr(stream, device)))
                 self._tensor_buf = buf
-            if not torch.cuda.is_current_stream_capturing():
-                (stream if stream is not None else torch.cuda.current_stream(device)).synchronize()
+            used = stream if stream is not None else torch.cuda.current_stream(device)
+            with torch.cuda.stream(used):
+                capturing = torch.cuda.is_current_stream_capturing()
+            if not capturing:
+                used.synchronize()
         return self
 
     def out_shape(self, x_shape) -> tuple:

@@ -110,3 +110,12 @@ def test_complete_on_return_whatever_the_layer_holds(fake):
         fake.calls.clear()
         layer.bind("cuda")
         assert [c[0] for c in fake.calls] == ["image"] + ["tensor"] * builds + ["done"]
+
+
+@pytest.mark.parametrize("capturing", ["given", "current"])
+def test_a_stream_under_capture_is_not_synchronised(fake, capturing):
+    """What counts is the stream that the work goes to, current or not."""
+    side = _Stream(0, capturing=capturing == "given")
+    fake.streams[0].capturing = capturing == "current"
+    _dense().bind("cuda", stream=side)
+    assert [c[2] for c in fake.calls] == [side.cuda_stream] * (2 if capturing == "given" else 3)
