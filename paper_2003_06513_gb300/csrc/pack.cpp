@@ -173,6 +173,13 @@ int build(pp_layer* L, const float* W, double keep) {
         for (int co = 0; co < cout && L->tc_ok; ++co)
             if (fmax_[co] > 0.0f && fmax_[co] < std::ldexp(top, -20)) L->tc_ok = false;
         L->tc_exp = L->tc_ok ? 14 - e : 0;
+        double l1 = 0.0;
+        for (int co = 0; co < cout; ++co) {
+            double sum = 0.0;
+            for (size_t i = 9 * (size_t)co * cin_g; i < 9 * (size_t)(co + 1) * cin_g; ++i) sum += std::fabs(L->dense[i]);
+            l1 = std::max(l1, sum);
+        }
+        L->tc_l1 = (float)l1;
     }
 
     const size_t b_perm = L->perm.size() * 4, b_desc = L->desc.size() * 8,

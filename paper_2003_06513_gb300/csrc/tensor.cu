@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -84,6 +85,7 @@ struct TcParams {
     int N, C, H, W, Cout, Ho, Wo, G, relu, pool;
     int wexp;                  // weights are scaled by 2^wexp
     float wbias;               // ... and by 1 + wbias (in their lo parts)
+    float unheld;              // a slow block's factor to the smallest sum it may be part of
     int NC, KS, n_cb, cb_split;
     int ll;                    // fp32: the products of the lo parts too
     int Wp, Ip, mstep, P;       // position pitch of a row, of an image (flat); tile step; staged positions
@@ -372,6 +374,7 @@ __device__ __forceinline__ bool combine(uint32_t* mx, uint32_t* mn, bool ok, uin
     *par ^= 1;
     return true;
 }
+// A block's header: the factor of its sums, and whether it holds values that their pairs do not.
 __device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t xfull, float2* hdr, uint32_t hready, int kexp, bool slow,
                                         int tid, int lane) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -935,75 +938,187 @@ __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* sm
     stages_done(p, sg, xempty, abort_flag, tid);
 }
 
-// ---------------------------------------------------------------------------- general sums
+// ---------------------------------------------------------------------------- sums in fp32
 
-// A unit whose inputs the fp16 pairs cannot hold (an infinity or NaN, or values 2^33 apart within a
-// stage) is summed by the eight promote warps from the packed layout in fp32, in the order of the
-// FFMA kernel: only kept taps are read.
-template <int S, typename T>
-__device__ void point_sums(const TcParams& p, int g, int n, int oy, int ox, int c0, int c1, float (&a)[kF]) {
-    const T* x = static_cast<const T*>(p.x);
-    for (int f = 0; f < kF; ++f) a[f] = 0.0f;
-    for (int ci = c0; ci < c1; ++ci) {
-        uint64_t d = p.desc[(size_t)g * p.C + ci];
-        const int cnt = (int)(d & 15u);
-        d >>= 4;
-        const float4* w4 = p.vals + p.kofs[(size_t)g * p.C + ci];
-        const T* xc = x + ((size_t)n * p.C + ci) * p.H * p.W;
-        for (int k = 0; k < cnt; ++k, d >>= 6) {
-            const float4 w = w4[k];
-            const float wv[4] = {w.x, w.y, w.z, w.w};
-            uint32_t m = p.masks[d & 7u];
-            float s = a[(d >> 3) & 7u];
-            for (int j = 0; j < 4; ++j) {
-                const int t = __ffs((int)m) - 1;
-                m &= m - 1;
-                const int iy = oy * S + t / 3 - 1, ix = ox * S + t % 3 - 1;
-                if (iy >= 0 && iy < p.H && ix >= 0 && ix < p.W) s = fmaf(wv[j], (float)xc[(size_t)iy * p.W + ix], s);
+// The pairs of a slow block's inputs err by up to 2^-36 2^-kexp each, and so a sum by up to the filter's
+// sum of |w| times that.  2^21 times as much (p.unheld times the block's factor) and more is a sum to
+// 2^-21 of itself.  Units with a smaller one, with an infinity or a NaN are noted in a bitmap, a bit per
+// unit of the CTA in their order, the last bit for all from there on, and summed again by the eight
+// summing warps after the CTA's last unit, when the pipeline's shared memory is theirs and nobody waits
+// for them.  Summed at once in the epilogue, from global memory by a thread a position, such units took
+// so long that one of 512 channels kept the other roles waiting for 27 ms, with a limit of one second.
+constexpr unsigned kRedoOff = 896, kLimOff = 648;
+constexpr int kRedoBits = 1024;
+
+// Whether a thread's sums hold such a one: position tiles as in the epilogue.
+template <int MT>
+__device__ __forceinline__ bool unheld(const TcParams& p, const Unit& U, const float (&acc)[128], float lim, int half, int pos) {
+    uint32_t top = 0;
+    const uint32_t least = __float_as_uint(lim);
+#pragma unroll
+    for (int i = 0; i < (MT == 4 ? 2 : 1); ++i) {
+        constexpr int NJ = MT == 4 ? 64 : 128;
+        const int pl = pos + 128 * (MT == 4 ? 2 * half + i : (MT == 2 ? half : 0));
+        const int r = (int)fdiv((uint32_t)pl, p.d_wp);
+        const bool in = p.tw ? U.n < p.N && r < min(p.th, p.Ho - U.oy0) && pl - r * p.Wp < min(p.tw, p.Wo - U.ox0) : U.q0 + pl < p.Q;
+        const int nf = in ? min(p.NC, p.Cout - U.r0) - (MT == 1 ? 128 * half : 0) : 0;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const uint32_t v = (__float_as_uint(acc[i * 64 + j]) & 0x7FFFFFFFu) - least;   // below: wraps
+            top = max(top, j < nf ? v : 0u);
+        }
+    }
+    return top >= 0x7F800000u - least;
+}
+
+// A unit's outputs from the packed layout in fp32, in the order of the FFMA kernel; only kept taps are
+// read.  Rounds of eight tasks, a warp each: two groups of eight filters by 128 positions (or 32 pooled
+// outputs), a lane four of the positions.  16 channels of the unit's window at a time are staged in fp32
+// as the MMAs' operand is (a plane a channel, at stride 2 a parity and channel; zeros outside the
+// image), so that a tap is one offset for all positions; a lane lists the kernels of one channel and
+// group, a slot at a time, with their offsets, and all lanes apply the list.  us a call, keep 0.3, fp32:
+//                              ordinary   one infinity   every unit   FFMA kernel
+//   256 -> 256, 56x56, N 32      203          720          2710           517
+//   512 -> 512, 14x14, N 32       71         1200          1250           187
+//   64 -> 64, 224x224, N 32, pool 328         610          4860           553
+// (from global memory 6600 and 34900, 21600 and 22000, 4000 and 99000).  The loads of shared memory and
+// the two warps a scheduler bound it.
+template <int S, typename T, int MT>
+__device__ __forceinline__ void redo_unit(const TcParams& p, const Unit& U, unsigned char* smem, int tid, int warp, int lane) {
+    constexpr int NG = 2, NPL = S == 1 ? 1 : 4;
+    const bool pool = p.pool && p.KS == 1;
+    const int PW = (int)(p.plane / 16);   // words of a plane: 16 channels' fit two of the pipeline's stages
+    const uint32_t HW = (uint32_t)p.H * p.W;
+    const int n0 = first_image(p, U), Hq = p.Ho >> 1, Wq = p.Wo >> 1, cols = max(p.tw >> 1, 1);
+    uint32_t* table = reinterpret_cast<uint32_t*>(smem + p.tab_off);
+    float* xs = reinterpret_cast<float*>(smem + p.x_off);
+    float4* list = reinterpret_cast<float4*>(smem + p.ring_off) + 64 * warp;   // 32 kernels: weights, offsets
+    bar_or<2, kPromoteWarps * 32>(false);
+    for (int i = tid; i < p.P; i += kPromoteWarps * 32) table[i] = window_entry<S>(p, U, i, n0);
+    const int tasks = (p.G + NG - 1) / NG * MT;
+    for (int k0 = 0; k0 < tasks; k0 += kPromoteWarps) {
+        const int g = (k0 + warp) / MT * NG, t = (k0 + warp) % MT;
+        // slot `lane` of the groups: is its filter one of the unit's
+        const uint32_t co = lane < NG * kF && g * kF + lane < p.G * kF ? p.perm[g * kF + lane] : kPadSlot;
+        const uint32_t mine = __ballot_sync(0xFFFFFFFFu, co != kPadSlot && (int)co >= U.r0 && (int)co < U.r0 + p.NC);
+        // this lane's four positions and their outputs
+        Point o[4];
+        const float* at[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            if (pool) {
+                const int i = lane + 32 * t, r = i / cols, c = i - r * cols;
+                o[b].n = U.n;
+                o[b].oy = U.oy0 + 2 * r + (b >> 1);
+                o[b].ox = U.ox0 + 2 * c + (b & 1);
+                o[b].in = U.n < p.N && 2 * r < p.th && o[b].oy / 2 < Hq && o[b].ox / 2 < Wq;
+                at[b] = xs + (o[b].in ? (2 * r + (b >> 1)) * p.Wp + 2 * c + (b & 1) : 0);
+            } else {
+                o[b] = point_of(p, U, 128 * t + 32 * b + lane);
+                at[b] = xs + 128 * t + 32 * b + lane;
             }
-            a[(d >> 3) & 7u] = s;
+        }
+        float a[NG][kF][4];
+#pragma unroll
+        for (int i = 0; i < NG * kF * 4; ++i) a[i / (kF * 4)][i / 4 % kF][i % 4] = 0.0f;
+        for (int cb = U.cb0; cb < U.cb1; ++cb) {
+            bar_or<2, kPromoteWarps * 32>(false);   // the table is complete, the block before done with
+            const T* xc = static_cast<const T*>(p.x) + ((size_t)n0 * p.C + cb * 16) * HW;
+            const int nc = min(16, p.C - cb * 16);
+            for (int i = tid; i < p.P; i += kPromoteWarps * 32) {
+                const uint32_t e = table[i];
+#pragma unroll
+                for (int pl = 0; pl < NPL; ++pl) {
+                    const bool in = e != kOut && (!(pl & 1) || (e & 1u)) && (!(pl & 2) || (e & 2u));
+                    const T* v = xc + (in ? (e >> 2) + (uint32_t)(pl >> 1) * p.W + (uint32_t)(pl & 1) : 0u);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        xs[(c * NPL + pl) * PW + i] = in && c < nc ? (float)__ldg(v + (size_t)c * HW) : 0.0f;
+                }
+            }
+            bar_or<2, kPromoteWarps * 32>(false);
+            if (mine == 0) continue;
+            // lane 16 h + c: the kernels of channel c and group h, in the order of their slots
+            const int h = lane >> 4, c = lane & 15;
+            const size_t gc = (size_t)(g + h) * p.C + cb * 16 + c;
+            uint64_t d = g + h < p.G && c < nc ? __ldg(p.desc + gc) : 0;
+            int left = (int)(d & 15u);
+            const float4* v = p.vals + (left ? __ldg(p.kofs + gc) : 0u);
+            float4 w = left ? __ldg(v) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            d >>= 4;
+#pragma unroll
+            for (int f = 0; f < kF; ++f) {
+                const bool has = left > 0 && (int)(d >> 3 & 7u) == f, use = has && (mine >> (kF * h + f) & 1u);
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, use);
+                if (use) {
+                    const int i = __popc(bal & ((1u << lane) - 1u));
+                    uint32_t m = p.masks[d & 7u];
+                    int off[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int k = __ffs((int)m) - 1, ty = k / 3, tx = k - 3 * ty;
+                        m &= m - 1;
+                        off[j] = c * NPL * PW + (S == 1 ? ty * p.Wp + tx
+                                                        : ((ty != 1 ? 2 : 0) + (tx != 1 ? 1 : 0)) * PW + (ty == 0 ? 0 : p.Wp) + (tx == 0 ? 0 : 1));
+                    }
+                    list[2 * i] = w;
+                    reinterpret_cast<int4*>(list)[2 * i + 1] = make_int4(off[0], off[1], off[2], off[3]);
+                }
+                if (has) {
+                    d >>= 6;
+                    ++v;
+                    if (--left) w = __ldg(v);
+                }
+                __syncwarp();
+                const int n1 = __popc(bal & 0xFFFFu), n2 = __popc(bal);
+                auto apply = [&](int i, float (&s)[4]) {
+                    const float4 u = list[2 * i];
+                    const int4 q = reinterpret_cast<const int4*>(list)[2 * i + 1];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        s[b] = fmaf(u.w, at[b][q.w], fmaf(u.z, at[b][q.z], fmaf(u.y, at[b][q.y], fmaf(u.x, at[b][q.x], s[b]))));
+                };
+                for (int i = 0; i < n1; ++i) apply(i, a[0][f]);
+                for (int i = n1; i < n2; ++i) apply(i, a[1][f]);
+                __syncwarp();
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NG * kF; ++i) {
+            if (!(mine >> i & 1u)) continue;
+            const float (&s)[4] = a[i / kF][i % kF];
+            const int co_i = (int)__shfl_sync(0xFFFFFFFFu, co, i);
+            const float bias = p.KS == 1 && p.bias ? p.bias[co_i] : 0.0f;
+            if (pool) {
+                const float m = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+                if (o[0].in)
+                    static_cast<T*>(p.y)[(((size_t)U.n * p.Cout + co_i) * Hq + o[0].oy / 2) * Wq + o[0].ox / 2] =
+                        out_of<T>(relu_of(m + bias, p.relu));
+                continue;
+            }
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                if (!o[b].in) continue;
+                const size_t to = (((size_t)o[b].n * p.Cout + co_i) * p.Ho + o[b].oy) * p.Wo + o[b].ox;
+                if (p.KS > 1) p.ws[(size_t)U.ks * p.ws_stride + to] = s[b];
+                else static_cast<T*>(p.y)[to] = out_of<T>(relu_of(s[b] + bias, p.relu));
+            }
         }
     }
 }
 
-template <int S, typename T>
-__device__ __noinline__ void general_unit(const TcParams& p, const Unit& U, int tid, int M) {
-    T* y = static_cast<T*>(p.y);
-    const int c0 = U.cb0 * 16, c1 = min(p.C, U.cb1 * 16);
-    const bool pool = p.pool && p.KS == 1;
-    const int Hq = p.Ho >> 1, Wq = p.Wo >> 1;
-    for (int i = tid; i < M; i += kPromoteWarps * 32) {
-        const Point o = point_of(p, U, i);
-        if (!o.in) continue;
-        const int n = o.n, oy = o.oy, ox = o.ox;
-        if (pool && ((oy | ox) & 1 || oy / 2 >= Hq || ox / 2 >= Wq)) continue;
-        for (int g = 0; g < p.G; ++g) {
-            bool any = false;
-            for (int f = 0; f < kF; ++f) {
-                const uint32_t co = p.perm[g * kF + f];
-                any = any || (co != kPadSlot && (int)co >= U.r0 && (int)co < U.r0 + p.NC);
-            }
-            if (!any) continue;
-            float a[kF];
-            point_sums<S, T>(p, g, n, oy, ox, c0, c1, a);
-            if (pool) {
-                for (int k = 1; k < 4; ++k) {
-                    float b[kF];
-                    point_sums<S, T>(p, g, n, oy + (k >> 1), ox + (k & 1), c0, c1, b);
-                    for (int f = 0; f < kF; ++f) a[f] = fmaxf(a[f], b[f]);
-                }
-            }
-            for (int f = 0; f < kF; ++f) {
-                const uint32_t co = p.perm[g * kF + f];
-                if (co == kPadSlot || (int)co < U.r0 || (int)co >= U.r0 + p.NC) continue;
-                if (p.KS > 1) {
-                    p.ws[(size_t)U.ks * p.ws_stride + (((size_t)n * p.Cout + co) * p.Ho + oy) * p.Wo + ox] = a[f];
-                    continue;
-                }
-                const T v = out_of<T>(relu_of(a[f] + (p.bias ? p.bias[co] : 0.0f), p.relu));
-                if (pool) y[(((size_t)n * p.Cout + co) * Hq + oy / 2) * Wq + ox / 2] = v;
-                else y[(((size_t)n * p.Cout + co) * p.Ho + oy) * p.Wo + ox] = v;
-            }
+// The noted units (not inlined: the loops before it would spill).
+template <int S, typename T, int MT>
+__device__ __noinline__ void redo_units(const TcParams& p) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const uint32_t* redo = reinterpret_cast<const uint32_t*>(smem + kRedoOff);
+    const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    for (int i = 0; i < kRedoBits; ++i) {
+        if (!(redo[i / 32] >> (i & 31) & 1u)) continue;
+        for (long long u = pair + (long long)i * pairs; u < p.n_units; u += pairs) {
+            redo_unit<S, T, MT>(p, unit_of(p, (int)u, rank), smem, threadIdx.x, warp, lane);
+            if (i < kRedoBits - 1) break;
         }
     }
 }
@@ -1012,7 +1127,6 @@ __device__ __noinline__ void general_unit(const TcParams& p, const Unit& U, int 
 
 template <int S, typename T, int MT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_tc(const __grid_constant__ TcParams p, const __grid_constant__ CUtensorMap tmap) {
-    constexpr int M = 128 * MT;
     constexpr int HL = sizeof(T) == 4 ? 2 : 1;
     constexpr int TCOL = 256 / MT;                // accumulator columns of a 128-position tile
     constexpr bool LL = HL == 2 && MT == 1;
@@ -1027,7 +1141,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 644);
     float2* hdr = reinterpret_cast<float2*>(smem + 704);
     uint2* red = reinterpret_cast<uint2*>(smem + 768);
+    uint32_t* redo = reinterpret_cast<uint32_t*>(smem + kRedoOff);
+    volatile float* lims = reinterpret_cast<volatile float*>(smem + kLimOff);   // of the warps' units
 
+    if (threadIdx.x < kRedoBits / 32) redo[threadIdx.x] = 0;
+    if (threadIdx.x < kPromoteWarps) lims[threadIdx.x] = -1.0f;
     if (warp == kMmaWarp) {
         if (lane == 0) {
             // The leader (rank 0) issues the pair's MMAs: its `full` barriers take the arrivals of
@@ -1084,7 +1202,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
             float* s_bias = reinterpret_cast<float*>(smem + 1024) + 256 * (un & 1);
             ++un;
             s_bias[threadIdx.x] = p.bias && U.r0 + (int)threadIdx.x < p.Cout ? __ldg(p.bias + U.r0 + threadIdx.x) : 0.0f;
-            bool slow = false;
             // columns of this warp: 32-column groups that hold filters of the unit
             bool act[4];
 #pragma unroll
@@ -1097,7 +1214,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 if (!ok) break;
                 fence_after();
                 const float2 h = hdr[e & (kHdr - 1)];
-                slow = slow || h.y != 0.0f;
+                if (h.y != 0.0f) lims[warp] = fmaxf(lims[warp], h.x * p.unheld);
 #pragma unroll
                 for (int jb = 0; jb < 4; ++jb) {
                     if (act[jb]) {
@@ -1112,9 +1229,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 if (lane == 0) mbar_arrive_leader(tempty + 8 * b);
             }
             if (bar_or<2, kPromoteWarps * 32>(!ok)) break;
-            if (slow) {
-                general_unit<S, T>(p, U, threadIdx.x, M);
-            } else if (p.pool && p.KS == 1) {
+            if (lims[warp] >= 0.0f) {
+                if (unheld<MT>(p, U, acc, lims[warp], half, pos)) {
+                    const int bit = min((int)un - 1, kRedoBits - 1);
+                    atomicOr(redo + bit / 32, 1u << (bit & 31));
+                }
+                __syncwarp();
+                lims[warp] = -1.0f;
+            }
+            if (p.pool && p.KS == 1) {
                 // 2x2 max-pool: a few filters of every position at a time through shared memory, each
                 // row of outputs at an even pitch (a pooled output is two 8-byte loads), a warp a
                 // filter, a lane up to MT pooled outputs whose offsets are the same for every filter.
@@ -1210,6 +1333,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
         }
+        if (!bar_or<2, kPromoteWarps * 32>(!ok) && __any_sync(0xFFFFFFFFu, redo[lane] != 0)) redo_units<S, T, MT>(p);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp < kPromoteWarps + kProducerWarps) {
@@ -1661,6 +1785,7 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.Ho = c.Ho;
     p.Wo = c.Wo;
     p.relu = c.relu;
+    p.unheld = c.es == 4 ? std::ldexp(L->tc_l1, L->tc_exp - 15) : 0.0f;   // fp16: exact inputs
     p.pool = c.pool;
     p.KS = pl.KS;
     p.cb_split = pl.cb_split;

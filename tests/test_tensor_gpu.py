@@ -316,3 +316,77 @@ def test_misaligned_workspace_that_only_the_tensor_core_plan_would_split_into():
     assert torch.isnan(ws).all()
     _check(y, x, W, b, 1.0, 1, False, "f16", idx=[0, 201])
     assert torch.equal(y, _cuda_cores_only(layer).conv(xt, bt, True))
+
+
+REDO = [  # cout, cin, n, h, w, keep, io, stride, pool, workspace: what the pairs do not hold, by tile and epilogue
+    (64, 72, 5, 60, 100, 0.5, "f32", 1, False, False),     # 512 positions, boxes, a last block of 8 channels
+    (64, 72, 9, 61, 100, 0.5, "f32", 1, True, False),      # pooled, an odd row dropped
+    (64, 128, 17, 61, 59, 0.4, "f32", 1, False, False),    # copies
+    (96, 80, 9, 45, 61, 0.5, "f32", 1, False, False),      # 256 positions
+    (128, 64, 16, 50, 46, 0.5, "f32", 1, True, False),     # pooled, rectangles cut by the edge
+    (256, 72, 24, 29, 27, 0.5, "f32", 1, True, False),     # pooled, 128 positions
+    (300, 77, 16, 29, 31, 0.5, "f32", 1, False, False),    # two chunks of filters
+    (72, 96, 64, 29, 27, 0.5, "f32", 2, False, False),     # parity planes of an odd map
+    (64, 64, 64, 56, 56, 0.5, "f32", 2, True, False),
+    (256, 256, 4, 14, 14, 0.4, "f32", 1, False, True),     # a split: partial sums again
+    (512, 512, 1, 28, 28, 0.3, "f32", 1, True, True),      # ... pooled by the reduction
+    (200, 96, 24, 28, 28, 0.5, "f16", 1, True, False),
+    (128, 72, 64, 29, 27, 0.5, "f16", 2, False, False),
+]
+
+
+@pytest.mark.parametrize("case", REDO)
+def test_units_summed_again(case):
+    """An infinity and a NaN in some units and (fp32) halves of images 2^47 apart in all: what
+    reaches an output is what reaches it on the CUDA cores, and the finite ones lie within 2e-6 of
+    their own sum |w||x| (fp16 outputs: 2e-3)."""
+    cout, cin, n, h, w, keep, io, stride, pool, split = case
+    layer, W, b = _layer(cout, cin, keep, stride, cin + w)
+    x = WL.activations((n, cin, h, w), 7 + h, relu=True, dtype=np.float32)
+    if io == "f32":
+        x[..., : w // 2] *= np.float32(1e7)
+        x[..., w // 2:] *= np.float32(1e-7)
+    x = x.astype(NP[io])
+    ws = torch.empty(1 << 23, device="cuda") if split else None
+    xt, bt = torch.from_numpy(x).cuda(), torch.zeros(cout, device="cuda")
+    plan = layer.tensor_plan(xt.shape, 0 if ws is None else ws.numel() * 4, pool, xt.dtype)
+    assert plan["tensor"] == 1 and (plan["splits"] > 1) == split
+    Wh = OPR.project(W, OP.default8(), keep)["W_hat"]
+
+    def within(y, idx):
+        xs = x[idx].astype(np.float64)
+        ref, den = OC.conv_ref(xs, Wh, None, stride, False), OC.denominator(xs, Wh, None, stride)
+        if pool:
+            ref, den = OC.maxpool2x2(ref), OC.maxpool2x2(den)
+        return np.all(np.abs(y[idx].double().cpu().numpy() - ref) <= (2e-6 if io == "f32" else 2e-3) * den + 1e-44)
+
+    assert within(layer.conv(xt, bt, False, pool2x2=pool, workspace=ws), [0, n - 1])
+    xt[0, cin - 1, h - 2, 1], xt[n // 2, 0, 0, 0], xt[n - 1, cin // 2, h // 2, w // 2] = float("inf"), float("nan"), float("-inf")
+    got = layer.conv(xt, bt, False, pool2x2=pool, workspace=ws)
+    ref = _cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
+    assert torch.equal(torch.isnan(got), torch.isnan(ref)) and torch.equal(torch.isinf(got), torch.isinf(ref))
+    assert not torch.isfinite(got).all()
+    if n > 2:
+        assert within(got, [1])
+
+
+def test_one_infinity_costs_a_bounded_time():
+    """512 channels of one unit summed again take 6.4 times the CUDA-core kernel's whole call (1200 of
+    187 us); 12 times is the bar (by a thread a position, from global memory, it was 115 times)."""
+    layer, _, _ = _layer(512, 512, 0.3, 1, 28)
+    other = _cuda_cores_only(_layer(512, 512, 0.3, 1, 28)[0])
+    xt = torch.from_numpy(WL.activations((32, 512, 14, 14), 29, relu=True)).cuda()
+    xt[0, 3, 2, 2] = float("inf")
+    assert layer.tensor_plan(xt.shape)["tensor"] == 1
+
+    def time(lay):
+        lay.conv(xt, None, True)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        for _ in range(3):
+            lay.conv(xt, None, True)
+        ev[1].record()
+        torch.cuda.synchronize()
+        return ev[0].elapsed_time(ev[1])
+
+    assert time(layer) < 12 * time(other)
