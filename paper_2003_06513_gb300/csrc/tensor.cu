@@ -8,8 +8,10 @@
 // rate, 60 at keep 1.
 //
 // Precision.  Every fp32 operand is held as two fp16 values, v = (h + l 2^-11) 2^-k with one
-// power of two k per layer (weights) or per stage (inputs: 16 channels of the staged positions),
-// so the pair carries 22 to 23 bits down to 2^-28 of the largest value.  A chain of MMAs first sums
+// power of two k per layer (weights) or per stage (inputs: 16 channels of the staged positions).  The
+// pair carries 22 to 23 bits of a scaled value down to 2^-14 and errs by 2^-36 below; an input stage's
+// largest is kept in [2^11, 2^15), the layer's largest weight in [2^14, 2^15).  Sums that smaller inputs
+// may have put off are found by a bound and taken again in fp32 (redo_unit).  A chain of MMAs first sums
 // the cross terms h_x l_w + l_x h_w of the nine taps, then adds h_x h_w with the accumulator scaled
 // by 2^-11 in the first of those MMAs (scale-input-d); the dropped l_x l_w is 2^-24.6 of a product
 // (rms), and tiles of one column block (MT 1: small batches, where the FFMA kernel's split sums round
@@ -670,7 +672,6 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                 if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
                 // hi parts up to 2^11 ... 2^15 use the pair's whole range; else the block is taken again
                 // (from memory), its largest value scaled to [2^13, 2^14)
-                int ex = (int)(mx >> 10) - 15 - kexp;
                 if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
                     int u1 = u;
                     asm volatile("" : "+r"(u1));   // the unit again: held in registers for this rare path it cost
@@ -699,7 +700,7 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                                 for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[a][j]));
                     }
                     if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return;
-                    ex = (int)(mx >> 24) - 127;
+                    const int ex = (int)(mx >> 24) - 127;
                     slow = ex < -60 || ex > 120;   // also infinities and NaN
                     if (!slow) {
                         kexp = 13 - ex;
@@ -711,7 +712,8 @@ __device__ __forceinline__ void produce_async(const TcParams& p, unsigned char* 
                         }
                     }
                 }
-                slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
+                // under 2^-15 a scaled value's pair errs by more than 2^-21 of it (2^-36)
+                slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 + kexp < -15);
             }
             publish(p, &sg, xfull, hdr, hready, kexp, slow, tid, lane);
         }
@@ -811,7 +813,6 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
             mx = max(b & 0xFFFFu, b >> 16);
             if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return drain();
             // as in produce_async: a block beyond the scale is taken again
-            int ex = (int)(mx >> 10) - 15 - kexp;
             bool slow = false;
             if (mn != 0xFFFFFFFFu && (mx < 0x6800u || mx >= 0x7800u)) {
                 mx = 0;
@@ -822,7 +823,7 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
                     for (int j = 0; j < 8; ++j) mx = max(mx, 2u * __float_as_uint(v[j]));
                 }
                 if (!combine<true>(&mx, &mn, ok, red, &sg.par, warp, lane)) return drain();
-                ex = (int)(mx >> 24) - 127;
+                const int ex = (int)(mx >> 24) - 127;
                 slow = ex < -60 || ex > 120;   // also infinities and NaN
                 if (!slow) {
                     kexp = 13 - ex;
@@ -836,7 +837,7 @@ __device__ __forceinline__ void produce_box(const TcParams& p, const CUtensorMap
                     bar_or<1, kProducers>(false);   // all have read the box
                 }
             }
-            slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 < ex - 33);
+            slow = slow || (mn != 0xFFFFFFFFu && (int)((mn + 1u) >> 24) - 127 + kexp < -15);
             ++done;
             if (++slot == p.rs) { slot = 0; ++ph; }
             if (tid == 0) issue();                  // into the stage just read

@@ -390,3 +390,28 @@ def test_one_infinity_costs_a_bounded_time():
         return ev[0].elapsed_time(ev[1])
 
     assert time(layer) < 12 * time(other)
+
+
+@pytest.mark.parametrize("below", [20, 24, 28, 30, 32, 36, 44])
+@pytest.mark.parametrize("w,boxes", [(36, 1), (38, 0)])
+def test_small_halves_beside_large_ones(w, boxes, below):
+    """Half of each row holds one constant, 2^-20 to 2^-44 of the other half's values, and the block
+    before leaves the scale at the low end of what is kept: outputs of the small half within 2e-6 of
+    their own sum |w||x|.  (The constant's bits are what its pair loses, the same way in every product.)"""
+    layer, W, _ = _layer(64, 64, 0.5, 1, 30)
+    rng = np.random.default_rng(31)
+    x = np.maximum(rng.standard_normal((33, 64, 42, w)), 0).clip(0, 3.9)
+    x[:, :16, ::3, 0] = 3.99                             # the first block's largest 2^1.99, the others' 2^-0.97
+    x[:, 16:] = x[:, 16:].clip(0, 0.51)
+    x[:, :16, :, w // 2:] = 0
+    x[:, 16:, :, w // 2:] = 1.2345678 * 2.0 ** -below
+    x = x.astype(np.float32)
+    xt = torch.from_numpy(x).cuda()
+    plan = layer.tensor_plan(xt.shape)
+    assert (plan["tensor"], plan["boxes"]) == (1, boxes)
+    got = layer.conv(xt, None, False)[[0, 32]].double().cpu().numpy()
+    Wh = OPR.project(W, OP.default8(), 0.5)["W_hat"]
+    xs = x[[0, 32]].astype(np.float64)
+    ref, den = OC.conv_ref(xs, Wh, None, 1, False), OC.denominator(xs, Wh, None, 1)
+    err = np.max(np.abs(got - ref) / den)
+    assert err <= 2e-6, f"{err:.2e}"
