@@ -54,6 +54,7 @@ struct pp_layer {
     bool tc_ok = false;                // the pairs hold every kept weight (pack.cpp)
     int tc_exp = 0;
     float tc_l1 = 0.0f;                // the largest sum of |w| of a filter
+    int tc_small = 0;                  // the most weights of a filter whose pairs do not hold them
     void* tdev = nullptr;              // caller-owned device buffer, built by pp_bind_tensor
 
     // launch plans by call shape (conv.cu), created on the first plan by call_once, so that calls

@@ -158,7 +158,8 @@ int build(pp_layer* L, const float* W, double keep) {
 
     // 6. may the tensor-core kernel hold the weights as fp16 pairs?  The pair of v 2^tc_exp, the
     // layer's largest weight in [2^14, 2^15), has 22 bits down to 2^-28 of that weight and an
-    // absolute error of 2^-50 of it below; a filter whose own largest weight is 2^-20 of the
+    // absolute error of 2^-50 of it below.  Weights whose pairs err by more than 2^-21 of them, under
+    // 2^-15 when scaled, are counted: the kernel then checks its sums against them.  A filter whose own largest weight is 2^-20 of the
     // layer's or less keeps the layer on the FFMA kernel, and so does a weight scale beyond
     // 2^+-30 (the scales of weights and inputs are divided out in fp32).
     L->tc_ok = false;
@@ -180,6 +181,13 @@ int build(pp_layer* L, const float* W, double keep) {
             l1 = std::max(l1, sum);
         }
         L->tc_l1 = (float)l1;
+        L->tc_small = 0;
+        for (int co = 0; co < cout; ++co) {
+            int n = 0;
+            for (size_t i = 9 * (size_t)co * cin_g; i < 9 * (size_t)(co + 1) * cin_g; ++i)
+                n += L->dense[i] != 0.0f && std::fabs(L->dense[i]) < std::ldexp(1.0f, -15 - L->tc_exp);
+            L->tc_small = std::max(L->tc_small, n);
+        }
     }
 
     const size_t b_perm = L->perm.size() * 4, b_desc = L->desc.size() * 8,

@@ -88,6 +88,7 @@ struct TcParams {
     int wexp;                  // weights are scaled by 2^wexp
     float wbias;               // ... and by 1 + wbias (in their lo parts)
     float unheld;              // a slow block's factor to the smallest sum it may be part of
+    int all_slow;              // weights that their pairs do not hold: every block
     int NC, KS, n_cb, cb_split;
     int ll;                    // fp32: the products of the lo parts too
     int Wp, Ip, mstep, P;       // position pitch of a row, of an image (flat); tile step; staged positions
@@ -383,7 +384,7 @@ __device__ __forceinline__ void publish(const TcParams& p, Stage* sg, uint32_t x
     __syncwarp();
     if (lane == 0 && !p.no_fill) mbar_arrive_leader(xfull + 8 * sg->s);
     if (tid == 0) {   // (the slot's header of kHdr blocks ago was read before this block's stage was freed)
-        hdr[sg->e & (kHdr - 1)] = make_float2(__uint_as_float((uint32_t)(127 - kexp - p.wexp) << 23), slow ? 1.0f : 0.0f);
+        hdr[sg->e & (kHdr - 1)] = make_float2(__uint_as_float((uint32_t)(127 - kexp - p.wexp) << 23), slow || p.all_slow ? 1.0f : 0.0f);
         mbar_arrive(hready + 8 * (sg->e & (kHdr - 1)));
     }
     ++sg->e;
@@ -1786,7 +1787,10 @@ cudaError_t tensor_launch(const TensorCall& c, const TensorPlan& pl) {
     p.Ho = c.Ho;
     p.Wo = c.Wo;
     p.relu = c.relu;
-    p.unheld = c.es == 4 ? std::ldexp(L->tc_l1, L->tc_exp - 15) : 0.0f;   // fp16: exact inputs
+    // fp32: the inputs' errors (redo_unit) and, of at most 2^15 2^-kexp each, the inputs at weights that
+    // err by 2^-36 2^-wexp; fp16: exact inputs of at most 2^16, and sums are rounded to 2^-12
+    p.unheld = c.es == 4 ? std::ldexp(L->tc_l1, L->tc_exp - 15) + (float)L->tc_small : std::ldexp((float)L->tc_small, -8);
+    p.all_slow = L->tc_small > 0;
     p.pool = c.pool;
     p.KS = pl.KS;
     p.cb_split = pl.cb_split;

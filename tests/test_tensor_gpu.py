@@ -415,3 +415,30 @@ def test_small_halves_beside_large_ones(w, boxes, below):
     ref, den = OC.conv_ref(xs, Wh, None, 1, False), OC.denominator(xs, Wh, None, 1)
     err = np.max(np.abs(got - ref) / den)
     assert err <= 2e-6, f"{err:.2e}"
+
+
+@pytest.mark.parametrize("io", ["f32", "f16"])
+@pytest.mark.parametrize("below", [24, 28, 32, 40, 56])
+def test_small_weights_beside_large_ones(below, io):
+    """One channel's weights are 2^-24 to 2^-56 of the others', and in half of each row that channel
+    alone has inputs: outputs there within 2e-6 of their own sum |w||x| (fp16 outputs, scaled into
+    range: 1e-3)."""
+    rng = np.random.default_rng(32)
+    W = (rng.standard_normal((64, 64, 3, 3)) * np.sqrt(2 / (9 * 64))).astype(np.float32)
+    W[:, 5] *= np.float32(2.0 ** -below)
+    x = np.maximum(rng.standard_normal((40, 64, 32, 32)), 0)
+    x[..., 16:] = 0
+    if io == "f16":
+        W *= np.float32(2.0 ** 24)
+        x[..., :16] *= 2.0 ** -24
+    x[:, 5, :, 16:] = 1.2345678
+    x = x.astype(NP[io])
+    layer = api.pp_pack(W, None, 1.0).bind("cuda")
+    xt = torch.from_numpy(x).cuda()
+    assert layer.tensor_plan(xt.shape, 0, False, xt.dtype)["tensor"] == 1
+    got = layer.conv(xt, None, False)[[0, 39]].double().cpu().numpy()
+    Wh = OPR.project(W, OP.default8(), 1.0)["W_hat"]
+    xs = x[[0, 39]].astype(np.float64)
+    ref, den = OC.conv_ref(xs, Wh, None, 1, False), OC.denominator(xs, Wh, None, 1)
+    err = np.max(np.abs(got - ref) / np.maximum(den, 1e-37 if io == "f32" else 6e-5))
+    assert err <= (2e-6 if io == "f32" else 1e-3), f"{err:.2e}"
