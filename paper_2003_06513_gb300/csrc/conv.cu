@@ -2657,7 +2657,8 @@ double shift_gain(double kept_per_channel) { return std::min(1.0, 0.82 + 0.0225 
 //                  schedule 1 + SMs / (2 units); 1.1 times that where it is not split
 //   tensor cores   1.0 + 0.033 blocks a split + 0.058 log2 splits + 0.5 (keep - 0.3), 0.84 for 1.0
 //                  with the lo products (the pairs alone are 0.7e-7); 0.25 more without them where
-//                  the FFMA plan has four splits or more, as what is compared is then small
+//                  the FFMA plan has four splits or more, as what is compared is then small; the square
+//                  of what the accumulator truncates where the weights don't carry it back
 // Below 13 products a piece the formula says too much of the FFMA kernel.  Over 150 drawn layers of 3
 // to 512 channels the error was above the FFMA kernel's in 3, by 4 % at most, before the last two
 // constants were raised for them.
@@ -2668,7 +2669,8 @@ bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int e
         const double ffma = (0.06 + 0.0137 * products / pieces + 0.036 * (pieces > 1.0 ? pieces : 0.0)) *
                             (pl.KS > 1 ? 1.0 : 1.1);
         const double tensor = (pl.tc.ll ? 0.84 : pl.KS >= 4 ? 1.25 : 1.0) + 0.033 * pl.tc.cb_split +
-                              0.058 * std::log2((double)pl.tc.KS) + 0.5 * std::max(0.0, keep - 0.3);
+                              0.058 * std::log2((double)pl.tc.KS) + 0.5 * std::max(0.0, keep - 0.3) +
+                              (L->tc_exact ? 1e14 * tensor_truncation(L) * tensor_truncation(L) : 0.0);
         if (products < 13.0 * pieces || tensor > ffma) return false;
     }
     if (!L->fast) return true;

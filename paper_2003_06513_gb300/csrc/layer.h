@@ -54,6 +54,7 @@ struct pp_layer {
     bool tc_ok = false;                // the pairs hold every kept weight (pack.cpp)
     int tc_exp = 0;
     float tc_l1 = 0.0f;                // the largest sum of |w| of a filter
+    bool tc_exact = false;             // every kept weight is one fp16 value
     int tc_small = 0;                  // the most weights of a filter whose pairs do not hold them
     void* tdev = nullptr;              // caller-owned device buffer, built by pp_bind_tensor
 

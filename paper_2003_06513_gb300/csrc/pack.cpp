@@ -161,7 +161,8 @@ int build(pp_layer* L, const float* W, double keep) {
     // absolute error of 2^-50 of it below.  Weights whose pairs err by more than 2^-21 of them, under
     // 2^-15 when scaled, are counted: the kernel then checks its sums against them.  A filter whose own largest weight is 2^-20 of the
     // layer's or less keeps the layer on the FFMA kernel, and so does a weight scale beyond
-    // 2^+-30 (the scales of weights and inputs are divided out in fp32).
+    // 2^+-30 (the scales of weights and inputs are divided out in fp32).  Weights that are fp16 values
+    // as they are (integers, powers of two) stay so: no bias is added to them (tensor_bias).
     L->tc_ok = false;
     if (!L->depthwise) {
         float top = 0.0f;
@@ -181,6 +182,12 @@ int build(pp_layer* L, const float* W, double keep) {
             l1 = std::max(l1, sum);
         }
         L->tc_l1 = (float)l1;
+        L->tc_exact = L->tc_ok;
+        for (size_t i = 0; i < 9 * K && L->tc_exact; ++i) {
+            uint32_t bits;
+            std::memcpy(&bits, &L->dense[i], 4);
+            L->tc_exact = (bits & 0x1FFFu) == 0 && (L->dense[i] == 0.0f || std::fabs(L->dense[i]) >= std::ldexp(1.0f, -14 - L->tc_exp));
+        }
         L->tc_small = 0;
         for (int co = 0; co < cout; ++co) {
             int n = 0;

@@ -17,7 +17,7 @@
 // (rms), and tiles of one column block (MT 1: small batches, where the FFMA kernel's split sums round
 // less) sum it as well.  The tensor core's accumulator truncates, so a chain covers 16 channels
 // only and the sums are then added in fp32 registers, rounded to nearest, by eight warps; what the
-// truncation takes away on average is put back into the weights (wbias below).
+// truncation takes away on average is put back into the weights (tensor_bias).
 // fp16 inputs are exact and need two products.
 //
 // Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 200,
@@ -1582,10 +1582,7 @@ void fill_layer(const pp_layer* L, TcParams* p) {
     p->NC = tensor_nc(L);
     p->n_cb = (L->cin_g + 15) / 16;
     p->wexp = L->tc_exp;
-    // A chain of nine accumulator truncations takes this share of its sum away on average; it grows
-    // with the kept share of the kernels (measured 0.8e-7 of the result at 0.3, 1.0e-7 at 0.5, 1.3e-7
-    // at 1).  The weights carry it back, in their lo parts.
-    p->wbias = 5.75e-8f + 7.5e-8f * (float)((double)L->beta / ((double)L->cout * L->cin_g));
+    p->wbias = (float)tensor_bias(L);
     for (int i = 0; i < kMaxPatterns; ++i) p->masks[i] = L->masks[i];
 }
 

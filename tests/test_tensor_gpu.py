@@ -442,3 +442,24 @@ def test_small_weights_beside_large_ones(below, io):
     ref, den = OC.conv_ref(xs, Wh, None, 1, False), OC.denominator(xs, Wh, None, 1)
     err = np.max(np.abs(got - ref) / np.maximum(den, 1e-37 if io == "f32" else 6e-5))
     assert err <= (2e-6 if io == "f32" else 1e-3), f"{err:.2e}"
+
+
+@pytest.mark.parametrize("cin,n,h,stride,split,io", [(256, 32, 28, 1, False, "f32"), (192, 32, 57, 2, False, "f32"),
+                                                     (256, 32, 28, 1, False, "f16"), (512, 1, 28, 1, True, "f16")])
+def test_integers_are_summed_exactly(cin, n, h, stride, split, io):
+    """Weights of a few bits and whole inputs, sums under 2^24: every output is the exact sum (fp16: its
+    rounding), as on the CUDA cores."""
+    rng = np.random.default_rng(33)
+    W = (rng.integers(-8, 9, (256, cin, 3, 3)) / 16).astype(np.float32)
+    x = rng.integers(0, 256 if io == "f32" else 16, (n, cin, h, h)).astype(NP[io])
+    layer = api.pp_pack(W, None, 0.4, 1, stride).bind("cuda")
+    xt = torch.from_numpy(x).cuda()
+    ws = torch.empty(1 << 23, device="cuda") if split else None
+    plan = layer.tensor_plan(xt.shape, 0 if ws is None else ws.numel() * 4, False, xt.dtype)
+    assert plan["tensor"] == 1 and (plan["splits"] > 1) == split
+    y = layer.conv(xt, None, False, workspace=ws)
+    Wh = OPR.project(W, OP.default8(), 0.4)["W_hat"]
+    idx = [0, n - 1] if n > 1 else [0]
+    ref = OC.conv_ref(x[idx].astype(np.float64), Wh, None, stride, False)
+    assert np.abs(ref).max() * 16 < 2 ** 24
+    assert np.array_equal(y[idx].cpu().numpy(), ref.astype(NP[io]))
