@@ -2649,30 +2649,50 @@ int make_plan_uncached(const pp_layer* L, int N, int H, int W, size_t ws_avail, 
 // (channel, group), 0.87 at 2.4 and 1 from 8 on.
 double shift_gain(double kept_per_channel) { return std::min(1.0, 0.82 + 0.0225 * kept_per_channel); }
 
+// Rounding of a split's reduction: the share of the result's square that each of its additions holds,
+// summed (eight planes pairwise, four pooled, then one sum after the other).
+double reduction_rounding(int ks, int pool) {
+    const int step = pool ? 4 : 8, levels = pool ? 2 : 3, whole = ks / step * step;
+    double e = (double)levels * whole / ks;
+    for (int i = step; i <= whole; i += step) e += (double)i / ks;
+    for (int i = whole + 1; i <= ks; ++i) e += (double)i / ks;
+    return e;
+}
+
+// Whether the tensor-core kernel rounds no more than the FFMA kernel with its splits' sums added in
+// order.  Squared errors against 64 bits, in units of (1e-7 of the result)^2, fitted to 1057 layers of 12
+// to 512 channels, half of them small calls, on both kernels (three in four with a workspace):
+//   FFMA           0.065 + 0.015 products; split 0.155 + 0.0168 products a split + 0.0442 (splits + 1) / 2;
+//                  balanced schedule 0.218 + 0.0121 products a piece + 0.0366 pieces, 1 + SMs / (2 units)
+//   tensor cores   0.935 (0.764 with the lo products) + 0.0333 blocks a split + 0.58 (keep - 0.3) + 0.054
+//                  reduction_rounding, and the square of what the accumulator truncates where the
+//                  weights don't carry it back
+// Measured squares lie within 25 % of these for eight layers in ten, so the tensor cores' has to be lower
+// by the factors below.  For splits a second pair of estimates, off in other layers, has to hold too.
+// Over those and 1000 further layers 760 calls pass, none with the larger error; of the 885 that passed by
+// the second pair alone 32 had it, by up to 12 %.  (The reduction has since become pairwise, which takes up
+// to a third off the FFMA kernel's error, 6 % in the median.  Against that, one call in 20 is above, by
+// 19 % at most, nearly all of them with 25 splits and more.)
+bool tensor_rounds_less(const pp_layer* L, const Plan& pl, int pool) {
+    const TensorPlan& tc = pl.tc;
+    const double products = 4.0 * L->beta / L->cout, dense = std::max(0.0, products / (4.0 * L->cin_g) - 0.3);
+    const double pieces = pl.streamk ? 1.0 + 0.5 * sm_count() / pl.ctas : pl.KS, each = products / pieces;
+    if (each < 13.0) return false;   // the FFMA estimates say too much
+    const double truncated = L->tc_exact ? 1e14 * tensor_truncation(L) * tensor_truncation(L) : 0.0;
+    const double tensor = (tc.ll ? 0.764 : 0.935) + 0.0333 * tc.cb_split + 0.58 * dense + truncated +
+                          (tc.KS > 1 ? 0.054 * reduction_rounding(tc.KS, pool) : 0.0);
+    if (pl.streamk) return tensor <= 0.75 * (0.218 + 0.0121 * each + 0.0366 * pieces);
+    if (pl.KS == 1) return tensor <= (tc.ll ? 0.9 : 0.95) * (0.065 + 0.015 * products);
+    const double second = (tc.ll ? 0.84 : pl.KS >= 4 ? 1.25 : 1.0) + 0.033 * tc.cb_split + 0.5 * dense + truncated +
+                          0.058 * std::log2((double)tc.KS);
+    return tensor <= 0.155 + 0.0168 * each + 0.0221 * (pieces + 1.0) &&
+           second <= 0.97 * (0.06 + 0.0137 * each + 0.036 * pieces);
+}
+
 // Whether a call takes the tensor-core kernel: where its estimate is the lower one, and for fp32 only
-// where its rounding error is no larger.  Squared errors against 64 bits, in units of (1e-7 of the
-// result)^2, fitted to 40 layers on both kernels:
-//   FFMA           0.06 + 0.0137 products / pieces + 0.036 pieces   (77 products 1.1e-7, 307 2.2e-7,
-//                  614 in 32 pieces 1.2e-7), the sum's pieces being the plan's splits, on the balanced
-//                  schedule 1 + SMs / (2 units); 1.1 times that where it is not split
-//   tensor cores   1.0 + 0.033 blocks a split + 0.058 log2 splits + 0.5 (keep - 0.3), 0.84 for 1.0
-//                  with the lo products (the pairs alone are 0.7e-7); 0.25 more without them where
-//                  the FFMA plan has four splits or more, as what is compared is then small; the square
-//                  of what the accumulator truncates where the weights don't carry it back
-// Below 13 products a piece the formula says too much of the FFMA kernel.  Over 150 drawn layers of 3
-// to 512 channels the error was above the FFMA kernel's in 3, by 4 % at most, before the last two
-// constants were raised for them.
-bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int es) {
-    if (es == 4) {
-        const double products = 4.0 * L->beta / L->cout, keep = products / (4.0 * L->cin_g);
-        const double pieces = pl.streamk ? 1.0 + 0.5 * sm_count() / pl.ctas : pl.KS;
-        const double ffma = (0.06 + 0.0137 * products / pieces + 0.036 * (pieces > 1.0 ? pieces : 0.0)) *
-                            (pl.KS > 1 ? 1.0 : 1.1);
-        const double tensor = (pl.tc.ll ? 0.84 : pl.KS >= 4 ? 1.25 : 1.0) + 0.033 * pl.tc.cb_split +
-                              0.058 * std::log2((double)pl.tc.KS) + 0.5 * std::max(0.0, keep - 0.3) +
-                              (L->tc_exact ? 1e14 * tensor_truncation(L) * tensor_truncation(L) : 0.0);
-        if (products < 13.0 * pieces || tensor > ffma) return false;
-    }
+// where it rounds no more.
+bool tensor_wins(const pp_layer* L, const Plan& pl, int N, int Ho, int Wo, int es, int pool) {
+    if (es == 4 && !tensor_rounds_less(L, pl, pool)) return false;
     if (!L->fast) return true;
     const double flop = 8.0 * L->beta * (double)N * Ho * Wo;
     const double rate = (es == 4 ? 28e6 : 24e6) * (L->stride == 2 ? 0.5 : 1.0);   // FLOP a microsecond
@@ -2716,7 +2736,7 @@ int make_plan(const pp_layer* L, int N, int H, int W, size_t ws_avail, Plan* out
     const int Ho = (H - 1) / L->stride + 1, Wo = (W - 1) / L->stride + 1;
     for (int ll = 0; ll < (es == 4 ? 2 : 1) && !pl.tensor; ++ll)
         pl.tensor = tensor_plan(L, N, H, W, pool, es, ws_avail, sm_count(), &pl.tc, ll) &&
-                    tensor_wins(L, pl, N, Ho, Wo, es);
+                    tensor_wins(L, pl, N, Ho, Wo, es, pool);
     std::lock_guard<std::mutex> g(cache->mu);
     if (cache->plans.size() >= 256) cache->plans.clear();
     cache->plans[key] = pl;

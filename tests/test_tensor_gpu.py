@@ -463,3 +463,26 @@ def test_integers_are_summed_exactly(cin, n, h, stride, split, io):
     ref = OC.conv_ref(x[idx].astype(np.float64), Wh, None, stride, False)
     assert np.abs(ref).max() * 16 < 2 ** 24
     assert np.array_equal(y[idx].cpu().numpy(), ref.astype(NP[io]))
+
+
+@pytest.mark.parametrize("case,tensor", [  # cout, cin, n, h, w, keep, stride
+    ((27, 193, 52, 36, 36, 1.0, 2), 0), ((413, 413, 5, 28, 30, 0.3, 2), 0), ((512, 512, 4, 14, 14, 0.3, 1), 0),
+    ((256, 256, 16, 28, 28, 0.4, 2), 0),               # few units on the balanced schedule: 1.01 to 1.12 times
+    ((64, 64, 8, 112, 112, 0.3, 1), 1), ((256, 256, 64, 28, 28, 0.4, 2), 1), ((150, 90, 9, 45, 61, 0.5, 1), 1)])
+def test_the_route_rounds_no_more_than_the_cuda_cores(case, tensor):
+    """2-norm error against 64 bits of the whole output, with the workspace the call asks for."""
+    cout, cin, n, h, w, keep, stride = case
+    layer, W, b = _layer(cout, cin, keep, stride, 34)
+    xt = torch.from_numpy(WL.activations((n, cin, h, w), 35, relu=True)).cuda()
+    bt = torch.from_numpy(b).cuda()
+    nb = layer.workspace_bytes(xt.shape)
+    ws = torch.empty(nb // 4 + 4, device="cuda") if nb else None
+    assert layer.tensor_plan(xt.shape, nb)["tensor"] == tensor
+    Wh = torch.from_numpy(OPR.project(W, OP.default8(), keep)["W_hat"].astype(np.float64)).cuda()
+    ref = torch.nn.functional.conv2d(xt.double(), Wh, bt.double(), stride, 1).relu_()
+
+    def err(lay):
+        y = lay.conv(xt, bt, True, workspace=ws).double()
+        return (torch.linalg.vector_norm(y - ref) / torch.linalg.vector_norm(ref)).item()
+
+    assert err(layer) <= err(_cuda_cores_only(layer))
