@@ -40,6 +40,19 @@ def lib():
     return _lib.load(build_if_missing=True)
 
 
+def cuda_cores_only(layer):
+    """Withdraw a bound layer's tensor-core weights (binding the device image again does), so that its
+    calls run on the CUDA cores by the plan that ``layer.plan`` reports."""
+    import ctypes
+    import torch
+    from paper_2003_06513_gb300 import _lib
+    buf = layer._dev_buf
+    _lib.check("pp_bind_device", _lib.load().pp_bind_device(
+        layer._h, ctypes.c_void_p(buf.data_ptr()), buf.numel(), None))
+    torch.cuda.synchronize()
+    return layer
+
+
 def cuda_ok():
     try:
         import torch

@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import cuda_cores_only
 from oracle import conv as OC
 from oracle import patterns as OP
 from oracle import project as OPR
@@ -45,12 +46,14 @@ def _np_dt(dt):
 
 
 def run_gpu(W, x, b, keep, stride=1, relu=True, depthwise=False, dtype=torch.float32, masks=None,
-            guard=0, to_host=True, ws=False, ws_bytes=None):
+            guard=0, to_host=True, ws=False, ws_bytes=None, cuda_cores=False):
     """Pack + bind + pp_conv; x host array; returns the output (host float64 unless
-    ``to_host=False``) and the layer."""
+    ``to_host=False``) and the layer.  ``cuda_cores``: without the tensor cores, by ``layer.plan``."""
     layer = api.pp_pack(W, masks, keep, W.shape[0] if depthwise else 1, stride)
     dev = torch.device("cuda")
     layer.bind(dev)
+    if cuda_cores:
+        cuda_cores_only(layer)
     xt = torch.from_numpy(np.ascontiguousarray(x)).to(dev)
     bt = None if b is None else torch.from_numpy(b).to(dev)
     shape = layer.out_shape(x.shape)
@@ -424,7 +427,7 @@ def test_conv_pool_fused_with_split_equals_unfused_pool():
     W, b = WL.weights(L), WL.bias(L)
     x = torch.from_numpy(WL.layer_input(L, 16)).cuda()
     bt = torch.from_numpy(b).cuda()
-    layer = api.pp_pack(W, None, L.keep).bind("cuda")
+    layer = cuda_cores_only(api.pp_pack(W, None, L.keep).bind("cuda"))
     nb = min(max(layer.workspace_bytes(x.shape, pool2x2=True), layer.workspace_bytes(x.shape)), SPLIT_CAP)
     assert layer.plan(x.shape, nb, pool2x2=True)["splits"] > 1
     ws = torch.full((nb // 4,), float("nan"), device="cuda")
@@ -470,13 +473,14 @@ def test_vgg16_chained_network_fused_pool():
     assert tuple(x.shape) == (2, 512, 7, 7)
 
 
-@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
-def test_back_to_back_layers_match_layers_run_one_at_a_time(dtype):
+@pytest.mark.parametrize("dtype,cuda_cores", [(torch.float32, True), (torch.float16, True), (torch.float16, False)])
+def test_back_to_back_layers_match_layers_run_one_at_a_time(dtype, cuda_cores):
     """Layers launched one after another on one stream with no synchronisation (each kernel may
     start its set-up while the previous one finishes) read exactly what the previous layer wrote:
     ping-pong buffers (so a layer overwrites what the layer before it read), one workspace shared
     by the split layers, a fused pool, a stride-2 layer and a depthwise layer; the chain, run three
-    times over, must equal the same layers run one at a time with a synchronisation after each."""
+    times over, must equal the same layers run one at a time with a synchronisation after each.
+    (fp32 stays on the CUDA cores here; in fp16 four of the layers take the tensor cores.)"""
     dev = torch.device("cuda")
     N = 2
     specs = [  # (Cin, Cout, H, stride, keep, depthwise, pool, input-channel split)
@@ -492,6 +496,8 @@ def test_back_to_back_layers_match_layers_run_one_at_a_time(dtype):
     for i, (ci, co, h, st, keep, dw, pool, _) in enumerate(specs):
         L = WL.ConvLayer(f"b2b{i}", ci, co, h, h, st, dw, keep, w_seed=900 + i, b_seed=950 + i)
         layers.append(api.pp_pack(WL.weights(L), None, keep, co if dw else 1, st).bind(dev))
+        if cuda_cores:
+            cuda_cores_only(layers[-1])
         biases.append(torch.from_numpy(WL.bias(L)).to(dev))
         in_shapes.append((N, ci, h, h))
         o = layers[-1].out_shape(in_shapes[-1])
@@ -542,9 +548,9 @@ def test_split_is_planned_for_small_images():
 
 def test_split_matches_oracle_single_pass_and_is_deterministic():
     L, W, b, x = _split_case()
-    y_split, lay = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=SPLIT_CAP)
-    y_split2, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=SPLIT_CAP)
-    y_one, _ = run_gpu(W, x, b, L.keep, ws=False)
+    y_split, lay = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=SPLIT_CAP, cuda_cores=True)
+    y_split2, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=SPLIT_CAP, cuda_cores=True)
+    y_one, _ = run_gpu(W, x, b, L.keep, ws=False, cuda_cores=True)
     assert np.array_equal(y_split, y_split2)
     ref, den = oracle(W, x[[0, 31]], b, L.keep)
     assert OC.max_norm_err(y_split[[0, 31]], ref, den) <= 1e-4
@@ -560,9 +566,9 @@ def test_balanced_schedule_copy_fallback_whole_images():
     L, W, b, x = _split_case()
     lay = api.pp_pack(W, None, L.keep)
     assert lay.plan(x.shape, lay.workspace_bytes(x.shape))["streamk"] == 1
-    y1, _ = run_gpu(W, x, b, L.keep, ws=True)
-    y2, _ = run_gpu(W, x, b, L.keep, ws=True)
-    y0, _ = run_gpu(W, x, b, L.keep, ws=False)
+    y1, _ = run_gpu(W, x, b, L.keep, ws=True, cuda_cores=True)
+    y2, _ = run_gpu(W, x, b, L.keep, ws=True, cuda_cores=True)
+    y0, _ = run_gpu(W, x, b, L.keep, ws=False, cuda_cores=True)
     assert np.array_equal(y1, y2)
     ref, den = oracle(W, x[[0, 31]], b, L.keep)
     assert OC.max_norm_err(y1[[0, 31]], ref, den) <= 1e-4
@@ -580,9 +586,9 @@ def test_balanced_schedule_matches_oracle_and_is_deterministic():
     lay = api.pp_pack(W, None, L.keep)
     pl = lay.plan(x.shape, lay.workspace_bytes(x.shape))
     assert pl["streamk"] == 1 and (pl["tile_by"], pl["tile_nb"]) == (1, 4)
-    y1, _ = run_gpu(W, x, b, L.keep, ws=True)
-    y2, _ = run_gpu(W, x, b, L.keep, ws=True)
-    y0, _ = run_gpu(W, x, b, L.keep, ws=False)
+    y1, _ = run_gpu(W, x, b, L.keep, ws=True, cuda_cores=True)
+    y2, _ = run_gpu(W, x, b, L.keep, ws=True, cuda_cores=True)
+    y0, _ = run_gpu(W, x, b, L.keep, ws=False, cuda_cores=True)
     assert np.array_equal(y1, y2)
     ref, den = oracle(W, x[[0, 31]], b, L.keep)
     assert OC.max_norm_err(y1[[0, 31]], ref, den) <= 1e-4
@@ -597,14 +603,14 @@ def test_split_with_small_workspace_and_fp16():
     out_bytes = 32 * 512 * 14 * 14 * 4
     assert need >= 2 * out_bytes
     # room for two splits only: still correct
-    y2, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=2 * out_bytes)
+    y2, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=2 * out_bytes, cuda_cores=True)
     ref, den = oracle(W, x[[5]], b, L.keep)
     assert OC.max_norm_err(y2[[5]], ref, den) <= 1e-4
     # too small for any split: single pass
-    y1, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=out_bytes)
+    y1, _ = run_gpu(W, x, b, L.keep, ws=True, ws_bytes=out_bytes, cuda_cores=True)
     assert OC.max_norm_err(y1[[5]], ref, den) <= 1e-4
     xh = x.astype(np.float16)
-    yh, _ = run_gpu(W, xh, b, L.keep, ws=True, dtype=torch.float16)
+    yh, _ = run_gpu(W, xh, b, L.keep, ws=True, dtype=torch.float16, cuda_cores=True)
     ref, den = oracle(W, xh[[3]], b, L.keep)
     assert OC.max_norm_err(yh[[3]], ref, den) <= 2e-3
 

@@ -2,7 +2,7 @@
 full batch.
 
 Each case states the plan outcome it exercises and asserts it through layer.plan (the same plan
-the launch uses): linear tiles, rectangles of several whole images, bands of block rows of
+the launch uses, the layer's tensor-core weights being withdrawn): linear tiles, rectangles of several whole images, bands of block rows of
 several images, the bank-group lane order,
 blocks shifted to start at output columns 4j - 1 (4j - 2 under the fp32 fused pool), the copy
 fallback for rows that are not a multiple of 16 bytes, fp16 stages through TMA without the fused
@@ -15,6 +15,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import cuda_cores_only
 from oracle import conv as OC
 from oracle import patterns as OP
 from oracle import project as OPR
@@ -36,7 +37,7 @@ def _run(cout, cin, n, h, w, keep, io, pool=False, stride=1, seed=0, relu_in=Tru
     b = (rng.standard_normal(cout) * 0.1).astype(np.float32)
     x = WL.activations((n, cin, h, w), seed + 17, relu=relu_in,
                        dtype=np.float32 if io == "f32" else np.float16)
-    layer = api.pp_pack(W, None, keep, 1, stride).bind("cuda")
+    layer = cuda_cores_only(api.pp_pack(W, None, keep, 1, stride).bind("cuda"))
     xt = torch.from_numpy(x).cuda()
     nb = layer.workspace_bytes(xt.shape, pool, xt.dtype)
     if ws_cap is not None:

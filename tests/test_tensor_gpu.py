@@ -13,6 +13,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import cuda_cores_only
 from oracle import conv as OC
 from oracle import patterns as OP
 from oracle import project as OPR
@@ -38,15 +39,6 @@ def _layer(cout, cin, keep, stride, seed, patterns=None):
     W = (rng.standard_normal((cout, cin, 3, 3)) * np.sqrt(2 / (9 * cin))).astype(np.float32)
     b = (rng.standard_normal(cout) * 0.1).astype(np.float32)
     return api.pp_pack(W, patterns, keep, 1, stride).bind("cuda"), W, b
-
-
-def _cuda_cores_only(layer):
-    """Binding the device image again withdraws the tensor cores."""
-    buf = layer._dev_buf
-    _lib.check("pp_bind_device", _lib.load().pp_bind_device(
-        layer._h, ctypes.c_void_p(buf.data_ptr()), buf.numel(), None))
-    torch.cuda.synchronize()
-    return layer
 
 
 def _check(y, x, W, b, keep, stride, pool, io, masks=None, idx=None):
@@ -79,6 +71,10 @@ CASES = [  # cout, cin, n, h, w, keep, io, stride, pool
     (128, 64, 16, 50, 46, 0.5, "f32", 1, True),        # pool, rectangles cut by the edge
     (256, 72, 24, 29, 27, 0.5, "f32", 1, True),        # pool, odd map: last row and column dropped
     (64, 64, 64, 56, 56, 0.5, "f32", 2, True),         # pool at stride 2
+    (16, 32, 64, 28, 28, 1.0, "f32", 1, False),        # MMAs of 16 columns
+    (17, 64, 64, 28, 28, 1.0, "f32", 1, False),        # 32 filters of 17
+    (17, 256, 64, 56, 56, 1.0, "f32", 2, False),
+    (8, 64, 256, 56, 56, 1.0, "f16", 1, True),         # 16 filters of 8
     (256, 64, 16, 28, 28, 1.0, "f16", 1, False),
     (90, 70, 16, 45, 37, 0.5, "f16", 1, False),
     (128, 72, 64, 29, 27, 0.5, "f16", 2, False),
@@ -104,7 +100,7 @@ def test_tensor_kernel_matches_oracle(case):
 
 
 @pytest.mark.parametrize("case", [(512, 512, 1, 14, 14, 0.3, False), (512, 512, 1, 28, 28, 0.3, True),
-                                  (256, 256, 4, 14, 14, 0.4, False), (128, 256, 2, 16, 17, 0.5, False)])
+                                  (256, 512, 4, 14, 14, 0.4, False), (300, 400, 1, 13, 17, 1.0, False)])
 def test_tensor_split_of_the_input_channels(case):
     """Few tiles and a workspace: partial sums per channel range, with the products of the lo parts
     (the CUDA-core plan, itself split, rounds less than three products do), added by the reduction;
@@ -137,7 +133,7 @@ def _sides(layer, W, x, stride, relu=False):
     xt = torch.from_numpy(x).cuda()
     assert layer.tensor_plan(xt.shape)["tensor"] == 1
     a = layer.conv(xt, None, relu)
-    c = _cuda_cores_only(api.pp_pack(W, None, 0.5, 1, stride).bind("cuda")).conv(xt, None, relu)
+    c = cuda_cores_only(api.pp_pack(W, None, 0.5, 1, stride).bind("cuda")).conv(xt, None, relu)
     return a.double().cpu().numpy(), c.double().cpu().numpy()
 
 
@@ -209,7 +205,7 @@ def test_same_result_every_time():
 def test_cuda_core_kernel_without_tensor_binding(case):
     cout, cin, n, h, keep, io, pool, stride = case
     layer, W, b = _layer(cout, cin, keep, stride, 20 + h)
-    _cuda_cores_only(layer)
+    cuda_cores_only(layer)
     x = WL.activations((n, cin, h, h), 30 + h, relu=True, dtype=NP[io])
     xt = torch.from_numpy(x).cuda()
     nb = layer.workspace_bytes(xt.shape, pool, xt.dtype)
@@ -260,7 +256,7 @@ def test_tensor_kernel_takes_its_input_by_boxes(case):
     assert torch.equal(layer.conv(off, bt, True, pool2x2=pool), y)
     xt[n - 1, cin - 1, h - 1, w - 2] = float("inf")
     y = layer.conv(xt, bt, False, pool2x2=pool)
-    ref = _cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
+    ref = cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
     assert torch.equal(torch.isfinite(y), torch.isfinite(ref)) and not torch.isfinite(y).all()
 
 
@@ -315,7 +311,7 @@ def test_misaligned_workspace_that_only_the_tensor_core_plan_would_split_into():
     y = layer.conv(xt, bt, True, workspace=ws[1:])
     assert torch.isnan(ws).all()
     _check(y, x, W, b, 1.0, 1, False, "f16", idx=[0, 201])
-    assert torch.equal(y, _cuda_cores_only(layer).conv(xt, bt, True))
+    assert torch.equal(y, cuda_cores_only(layer).conv(xt, bt, True))
 
 
 REDO = [  # cout, cin, n, h, w, keep, io, stride, pool, workspace: what the pairs do not hold, by tile and epilogue
@@ -328,7 +324,7 @@ REDO = [  # cout, cin, n, h, w, keep, io, stride, pool, workspace: what the pair
     (300, 77, 16, 29, 31, 0.5, "f32", 1, False, False),    # two chunks of filters
     (72, 96, 64, 29, 27, 0.5, "f32", 2, False, False),     # parity planes of an odd map
     (64, 64, 64, 56, 56, 0.5, "f32", 2, True, False),
-    (256, 256, 4, 14, 14, 0.4, "f32", 1, False, True),     # a split: partial sums again
+    (256, 512, 4, 14, 14, 0.4, "f32", 1, False, True),     # a split: partial sums again
     (512, 512, 1, 28, 28, 0.3, "f32", 1, True, True),      # ... pooled by the reduction
     (200, 96, 24, 28, 28, 0.5, "f16", 1, True, False),
     (128, 72, 64, 29, 27, 0.5, "f16", 2, False, False),
@@ -363,7 +359,7 @@ def test_units_summed_again(case):
     assert within(layer.conv(xt, bt, False, pool2x2=pool, workspace=ws), [0, n - 1])
     xt[0, cin - 1, h - 2, 1], xt[n // 2, 0, 0, 0], xt[n - 1, cin // 2, h // 2, w // 2] = float("inf"), float("nan"), float("-inf")
     got = layer.conv(xt, bt, False, pool2x2=pool, workspace=ws)
-    ref = _cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
+    ref = cuda_cores_only(layer).conv(xt, bt, False, pool2x2=pool)
     assert torch.equal(torch.isnan(got), torch.isnan(ref)) and torch.equal(torch.isinf(got), torch.isinf(ref))
     assert not torch.isfinite(got).all()
     if n > 2:
@@ -374,7 +370,7 @@ def test_one_infinity_costs_a_bounded_time():
     """512 channels of one unit summed again take 6.4 times the CUDA-core kernel's whole call (1200 of
     187 us); 12 times is the bar (by a thread a position, from global memory, it was 115 times)."""
     layer, _, _ = _layer(512, 512, 0.3, 1, 28)
-    other = _cuda_cores_only(_layer(512, 512, 0.3, 1, 28)[0])
+    other = cuda_cores_only(_layer(512, 512, 0.3, 1, 28)[0])
     xt = torch.from_numpy(WL.activations((32, 512, 14, 14), 29, relu=True)).cuda()
     xt[0, 3, 2, 2] = float("inf")
     assert layer.tensor_plan(xt.shape)["tensor"] == 1
@@ -485,4 +481,4 @@ def test_the_route_rounds_no_more_than_the_cuda_cores(case, tensor):
         y = lay.conv(xt, bt, True, workspace=ws).double()
         return (torch.linalg.vector_norm(y - ref) / torch.linalg.vector_norm(ref)).item()
 
-    assert err(layer) <= err(_cuda_cores_only(layer))
+    assert err(layer) <= err(cuda_cores_only(layer))

@@ -16,6 +16,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import cuda_cores_only
 from oracle import conv as OC
 from oracle import patterns as OP
 from oracle import project as OPR
@@ -36,7 +37,8 @@ def _call_static(lib, layer, x, b, y, relu=1):
                                       ctypes.c_void_p(y.data_ptr()), None)
 
 
-def test_static_scratch_entry_point_matches_workspace_entry_point():
+@pytest.mark.parametrize("cuda_cores", [True, False])
+def test_static_scratch_entry_point_matches_workspace_entry_point(cuda_cores):
     lib = _lib.load()
     cap = ctypes.c_size_t()
     assert lib.pp_static_scratch_bytes(ctypes.byref(cap)) == 0 and cap.value == 32 << 20
@@ -45,9 +47,11 @@ def test_static_scratch_entry_point_matches_workspace_entry_point():
     W, bias = WL.weights(L), WL.bias(L)
     x_np = WL.layer_input(L, 16)
     layer = api.pp_pack(W, None, L.keep).bind("cuda")
+    if cuda_cores:
+        cuda_cores_only(layer)
     x = torch.from_numpy(x_np).cuda()
     b = torch.from_numpy(bias).cuda()
-    plan = layer.plan(x.shape, cap.value)             # the split the static call runs
+    plan = layer.plan(x.shape, cap.value)             # the split the static call runs on the CUDA cores
     need = plan["workspace_bytes"]
     assert plan["splits"] > 1 and 0 < need <= cap.value
 
