@@ -47,7 +47,7 @@ constexpr int kPromoteWarps = 8;        // warps 0-7: sums in registers, epilogu
 constexpr int kProducerWarps = 6;       // warps 8-13: input staging
 constexpr int kLoaderWarp = 14, kMmaWarp = 15;
 constexpr int kProducers = kProducerWarps * 32;
-constexpr int kMaxWSlots = 12, kMaxXStages = 4, kMaxRaw = 3;
+constexpr int kMaxWSlots = 6, kMaxXStages = 3, kMaxRaw = 2;   // as tensor_plan deals shared memory out
 // items a producer thread's copies run ahead, plus one, by the words of a channel in an item
 constexpr int ring_of(int words) { return words == 1 ? 6 : (words == 2 ? 4 : 3); }
 constexpr int kHdr = 8;                 // stage headers in flight
@@ -1710,24 +1710,24 @@ bool tensor_plan(const pp_layer* L, int N, int H, int W, int pool, int es, size_
             c.ring_off = (unsigned)align_up(c.tab_off + std::max<size_t>(4 * (size_t)c.P, 8 * (size_t)c.n_entries), 128);
             const int words = es == 4 ? vec : std::max(1, vec / 2);
             c.x_off = c.ring_off + std::max(ring_of(1) * 9, ring_of(words) * (8 * words + 1)) * kProducers * 4;
-            if (c.box) {   // two or three boxes; the copies' ring, should x not be aligned, in their place
+            if (c.box) {   // two boxes (three: no change); the copies' ring, should x not be aligned, in their place
                 c.rw = (3 + c.Wp + 3) & ~3;
                 const size_t box = (size_t)64 * (c.th + 2) * c.rw;
                 if (c.rw > 256 || c.th + 2 > 256) continue;
-                c.rs = 2;
+                c.rs = kMaxRaw;
                 c.x_off = (unsigned)(c.ring_off + std::max(align_up(c.rs * box, 128), (size_t)ring_of(1) * 9 * kProducers * 4));
             }
             if (c.x_off >= kSmemMax) continue;
             const size_t left = kSmemMax - c.x_off;
             // three input stages with two blocks' weights, else two with at least a block's and a row
             c.xs = 0;
-            for (int xs = 3; xs >= 2 && !c.xs; --xs) {
+            for (int xs = kMaxXStages; xs >= 2 && !c.xs; --xs) {
                 const int hs = xs == 3 ? 6 : 4, ls = 2;
                 if ((size_t)xs * c.x_stage + (size_t)(hs + ls) * c.w_slot > left) continue;
                 c.xs = xs;
                 const int slots = (int)std::min<size_t>(10, (left - (size_t)xs * c.x_stage) / c.w_slot);
                 c.ls = slots < 7 ? 2 : (slots < 10 ? 3 : 4);
-                c.hs = slots - c.ls;
+                c.hs = slots - c.ls;   // 4 to kMaxWSlots
             }
             if (!c.xs || (ll && c.ls < 3)) continue;   // a block's three rows of lo weights stay
             c.ll = ll;
