@@ -2663,16 +2663,17 @@ double reduction_rounding(int ks, int pool) {
 // order.  Squared errors against 64 bits, in units of (1e-7 of the result)^2, fitted to 1057 layers of 12
 // to 512 channels, half of them small calls, on both kernels (three in four with a workspace):
 //   FFMA           0.065 + 0.015 products; split 0.155 + 0.0168 products a split + 0.0442 (splits + 1) / 2;
-//                  balanced schedule 0.218 + 0.0121 products a piece + 0.0366 pieces, 1 + SMs / (2 units)
+//                  balanced schedule (360 further layers) 0.197 + 0.0147 products times the squares of the
+//                  shares that cut units' pieces have + 0.0536 of the additions' shares, over the units
 //   tensor cores   0.935 (0.764 with the lo products) + 0.0333 blocks a split + 0.58 (keep - 0.3) + 0.054
 //                  reduction_rounding, and the square of what the accumulator truncates where the
 //                  weights don't carry it back
 // Measured squares lie within 25 % of these for eight layers in ten, so the tensor cores' has to be lower
 // by the factors below.  For splits a second pair of estimates, off in other layers, has to hold too.
-// Over those and 1000 further layers 760 calls pass, none with the larger error; of the 885 that passed by
-// the second pair alone 32 had it, by up to 12 %.  (The reduction has since become pairwise, which takes up
-// to a third off the FFMA kernel's error, 6 % in the median.  Against that, one call in 20 is above, by
-// 19 % at most, nearly all of them with 25 splits and more.)
+// Of these layers and 1000 others 923 calls pass, none with the larger error (of the 885 that pass by the
+// second pair alone 32 had it, by up to 12 %); of 460 calls drawn afterwards one had, by 1.6 %.  (The reduction has since become pairwise, which takes up to a third off the FFMA kernel's error,
+// 6 % in the median.  Against that, one call in 20 is above, by 19 % at most, nearly all of them with 25
+// splits and more.)
 bool tensor_rounds_less(const pp_layer* L, const Plan& pl, int pool) {
     const TensorPlan& tc = pl.tc;
     const double products = 4.0 * L->beta / L->cout, dense = std::max(0.0, products / (4.0 * L->cin_g) - 0.3);
@@ -2681,7 +2682,29 @@ bool tensor_rounds_less(const pp_layer* L, const Plan& pl, int pool) {
     const double truncated = L->tc_exact ? 1e14 * tensor_truncation(L) * tensor_truncation(L) : 0.0;
     const double tensor = (tc.ll ? 0.764 : 0.935) + 0.0333 * tc.cb_split + 0.58 * dense + truncated +
                           (tc.KS > 1 ? 0.054 * reduction_rounding(tc.KS, pool) : 0.0);
-    if (pl.streamk) return tensor <= 0.75 * (0.218 + 0.0121 * each + 0.0366 * pieces);
+    if (pl.streamk) {
+        const long long sms = sm_count(), nck = pl.n_chunks, chunks = pl.ctas * nck;
+        double squares = (double)pl.ctas, adds = 0.0;
+        long long unit = -1, from = 0;   // the cut unit at hand, where its last piece ends
+        for (long long b = 1; b <= sms; ++b) {
+            const long long c = chunks * b / sms, u = c / nck, k = c - u * nck;
+            if (unit >= 0 && (u != unit || b == sms)) {
+                squares += (double)((nck - from) * (nck - from)) / (double)(nck * nck);
+                adds += 1.0;
+                unit = -1;
+            }
+            if (k == 0) continue;
+            if (unit < 0) {
+                unit = u;
+                from = 0;
+                squares -= 1.0;
+            }
+            squares += (double)((k - from) * (k - from)) / (double)(nck * nck);
+            if (from > 0 && k > from) adds += (double)k / nck;
+            from = k;
+        }
+        return tensor <= 0.93 * (0.197 + (0.0147 * products * squares + 0.0536 * adds) / (double)pl.ctas);
+    }
     if (pl.KS == 1) return tensor <= (tc.ll ? 0.9 : 0.95) * (0.065 + 0.015 * products);
     const double second = (tc.ll ? 0.84 : pl.KS >= 4 ? 1.25 : 1.0) + 0.033 * tc.cb_split + 0.5 * dense + truncated +
                           0.058 * std::log2((double)tc.KS);

@@ -949,7 +949,7 @@ __device__ __forceinline__ void produce_f16(const TcParams& p, unsigned char* sm
 // summing warps after the CTA's last unit, when the pipeline's shared memory is theirs and nobody waits
 // for them.  Summed at once in the epilogue, from global memory by a thread a position, such units took
 // so long that one of 512 channels kept the other roles waiting for 27 ms, with a limit of one second.
-constexpr unsigned kRedoOff = 896, kLimOff = 648;
+constexpr unsigned kRedoOff = 896;   // in shared memory
 constexpr int kRedoBits = 1024;
 
 // Whether a thread's sums hold such a one: position tiles as in the epilogue.
@@ -1144,10 +1144,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
     float2* hdr = reinterpret_cast<float2*>(smem + 704);
     uint2* red = reinterpret_cast<uint2*>(smem + 768);
     uint32_t* redo = reinterpret_cast<uint32_t*>(smem + kRedoOff);
-    volatile float* lims = reinterpret_cast<volatile float*>(smem + kLimOff);   // of the warps' units
 
     if (threadIdx.x < kRedoBits / 32) redo[threadIdx.x] = 0;
-    if (threadIdx.x < kPromoteWarps) lims[threadIdx.x] = -1.0f;
     if (warp == kMmaWarp) {
         if (lane == 0) {
             // The leader (rank 0) issues the pair's MMAs: its `full` barriers take the arrivals of
@@ -1204,19 +1202,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
             float* s_bias = reinterpret_cast<float*>(smem + 1024) + 256 * (un & 1);
             ++un;
             s_bias[threadIdx.x] = p.bias && U.r0 + (int)threadIdx.x < p.Cout ? __ldg(p.bias + U.r0 + threadIdx.x) : 0.0f;
+            float lim = -1.0f;
             // columns of this warp: 32-column groups that hold filters of the unit
             bool act[4];
 #pragma unroll
             for (int jb = 0; jb < 4; ++jb) act[jb] = ((128 * half + 32 * jb) % TCOL) < p.NC;
             for (int cb = U.cb0; cb < U.cb1 && ok; ++cb, ++e) {
                 const uint32_t b = e & 1u;
-                ok = wait_bar(hready + 8 * (e & (kHdr - 1)), (e / kHdr) & 1u, p, abort_flag, kErrData) &&
-                     wait_bar(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData);
+                const uint32_t hb = hready + 8 * (e & (kHdr - 1)), hp = (e / kHdr) & 1u;
+                const bool h1 = mbar_try(hb, hp), t1 = mbar_try(tfull + 8 * b, (e >> 1) & 1u);
+                ok = (h1 || wait_bar(hb, hp, p, abort_flag, kErrData)) &&
+                     (t1 || wait_bar(tfull + 8 * b, (e >> 1) & 1u, p, abort_flag, kErrData));
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
                 fence_after();
                 const float2 h = hdr[e & (kHdr - 1)];
-                if (h.y != 0.0f) lims[warp] = fmaxf(lims[warp], h.x * p.unheld);
+                lim = fmaxf(lim, h.y != 0.0f ? h.x * p.unheld : -1.0f);
 #pragma unroll
                 for (int jb = 0; jb < 4; ++jb) {
                     if (act[jb]) {
@@ -1231,13 +1232,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 if (lane == 0) mbar_arrive_leader(tempty + 8 * b);
             }
             if (bar_or<2, kPromoteWarps * 32>(!ok)) break;
-            if (lims[warp] >= 0.0f) {
-                if (unheld<MT>(p, U, acc, lims[warp], half, pos)) {
+            if (lim >= 0.0f) {
+                if (unheld<MT>(p, U, acc, lim, half, pos)) {
                     const int bit = min((int)un - 1, kRedoBits - 1);
                     atomicOr(redo + bit / 32, 1u << (bit & 31));
                 }
-                __syncwarp();
-                lims[warp] = -1.0f;
             }
             if (p.pool && p.KS == 1) {
                 // 2x2 max-pool: a few filters of every position at a time through shared memory, each
