@@ -147,8 +147,9 @@ int pp_bind_device(pp_handle h, void* dev_image, size_t bytes, void* stream);
  * on `stream`.  The same rules as for the image: the caller keeps the memory alive and unmodified
  * while the handle is used and orders this call before the first pp_conv.  The device of `dev` must
  * be the current one (a kernel builds the weights).  Later calls of pp_conv
- * and its variants then take the tensor-core kernel wherever it is the faster one; results agree
- * to fp32 rounding.  Without this call they run on the CUDA cores.  pp_bind_device withdraws it.
+ * and its variants then take the tensor-core kernel wherever it is the faster one and, in fp32, by
+ * estimate rounds no more: each output within 2e-6 of its own sum of |w||x|, whatever the inputs'
+ * range, infinities and NaN as on the CUDA cores.  Without this call they run on the CUDA cores.  pp_bind_device withdraws it.
  * Errors: PP_ERR_NULL, PP_ERR_NOT_BOUND, PP_ERR_PATH (PP_Q_TENSOR_BYTES is 0: depthwise layers and
  * weights of extreme range), PP_ERR_BUFFER (too small), PP_ERR_ALIGN, PP_ERR_CUDA. */
 int pp_bind_tensor(pp_handle h, void* dev, size_t bytes, void* stream);

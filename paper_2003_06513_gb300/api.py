@@ -97,8 +97,8 @@ class Layer:
     # ---- device side
     def bind(self, device=None, stream=None) -> "Layer":
         """Copy the device image into a fresh torch buffer on ``device`` and build the tensor-core
-        weights beside it where the layer has them (on ``stream``; complete on return, so that calls
-        on any stream may follow, unless the stream is being captured)."""
+        weights beside it where the layer has them (36 bytes a kernel, kept or not), on ``stream``;
+        waits for it, so that calls on any stream may follow, unless the stream is being captured."""
         device = torch.device(device if device is not None else "cuda")
         if device.type != "cuda":
             raise ValueError("the packed image must live in CUDA device memory")
@@ -133,8 +133,9 @@ class Layer:
 
     def plan(self, x_shape, workspace_bytes: int = 0, pool2x2: bool = False,
              dtype=torch.float32) -> dict:
-        """Launch plan pp_conv_ws (or, with pool2x2, pp_conv_pool_ws) would use for an input of
-        shape [N, C, H, W] and dtype (pp_conv_plan_dt).  Depthwise layers report ``dw_kernel``:
+        """Launch plan pp_conv_ws (or, with pool2x2, pp_conv_pool_ws) would use on the CUDA cores for an
+        input of shape [N, C, H, W] and dtype (pp_conv_plan_dt); a bound layer's call that takes the
+        tensor cores (``tensor_plan``) runs by that plan instead.  Depthwise layers report ``dw_kernel``:
         1 streamed rows, 2 streamed planes at stride 2, 3 / 4 streamed planes at stride 1 (rows of
         even / odd width), 5 / 6 streamed tiles of 7 / 14 columns at stride 1, 7 streamed tiles at
         stride 2, 0 the row-item kernels (for 16-byte aligned x and y)."""

@@ -2671,9 +2671,10 @@ double reduction_rounding(int ks, int pool) {
 // Measured squares lie within 25 % of these for eight layers in ten, so the tensor cores' has to be lower
 // by the factors below.  For splits a second pair of estimates, off in other layers, has to hold too.
 // Of these layers and 1000 others 923 calls pass, none with the larger error (of the 885 that pass by the
-// second pair alone 32 had it, by up to 12 %); of 460 calls drawn afterwards one had, by 1.6 %.  (The reduction has since become pairwise, which takes up to a third off the FFMA kernel's error,
-// 6 % in the median.  Against that, one call in 20 is above, by 19 % at most, nearly all of them with 25
-// splits and more.)
+// second pair alone 32 had it, by up to 12 %); of 460 calls drawn afterwards one had, by 1.6 %.  (The
+// reduction has since become pairwise, which takes up to a third off the FFMA kernel's error, 6 % in the
+// median.  Against that, one call in 20 is above, by 19 % at most, nearly all of them with 25 splits and
+// more.)
 bool tensor_rounds_less(const pp_layer* L, const Plan& pl, int pool) {
     const TensorPlan& tc = pl.tc;
     const double products = 4.0 * L->beta / L->cout, dense = std::max(0.0, products / (4.0 * L->cin_g) - 0.3);

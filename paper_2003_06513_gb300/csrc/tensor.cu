@@ -20,12 +20,12 @@
 // truncation takes away on average is put back into the weights (tensor_bias).
 // fp16 inputs are exact and need two products.
 //
-// Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 200,
-// 512->512 14x14 183 -> 70, 64->64 224x224 with the pool 547 -> 326, 256->256 28x28 stride 2
-// 200 -> 54; fp16 256->256 28x28 keep 1 808 -> 75.  What bounds it: 13 % over the bare MMA stream
-// (175 us) on the 56x56 and 28x28 layers of 256 and 512 filters, the input staging (six warps:
-// split into pairs, store) with 64 filters or stride 2, one partial wave of CTA pairs on the
-// smallest.
+// Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 202,
+// 512->512 14x14 183 -> 71, 64->64 224x224 with the pool 547 -> 328, 256->256 28x28 stride 2
+// 200 -> 55; fp16 256->256 28x28 keep 1 808 -> 75.  What bounds it: the MMA rate and the last wave
+// (56x56: 5.36 waves of CTA pairs run as 6; 72 % of the tensor pipe) on the 56x56 and 28x28 layers of
+// 256 and 512 filters, the input staging (six warps: split into pairs, store) with 64 filters or
+// stride 2, one partial wave on the smallest.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
