@@ -1232,13 +1232,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                 if (lane == 0) mbar_arrive_leader(tempty + 8 * b);
             }
             if (bar_or<2, kPromoteWarps * 32>(!ok)) break;
-            if (lim >= 0.0f) {
-                if (unheld<MT>(p, U, acc, lim, half, pos)) {
+            // before the pooled epilogue and after the other (all after: 64 -> 64 224x224 336 for 327 us; all
+            // before: 256 -> 256 56x56 202.5 for 201.6, 90 -> 150 45x61 20.0 for 19.4)
+            auto note_unheld = [&]() {
+                if (lim >= 0.0f && unheld<MT>(p, U, acc, lim, half, pos)) {
                     const int bit = min((int)un - 1, kRedoBits - 1);
                     atomicOr(redo + bit / 32, 1u << (bit & 31));
                 }
-            }
+            };
             if (p.pool && p.KS == 1) {
+                note_unheld();
                 // 2x2 max-pool: a few filters of every position at a time through shared memory, each
                 // row of outputs at an even pitch (a pooled output is two 8-byte loads), a warp a
                 // filter, a lane up to MT pooled outputs whose offsets are the same for every filter.
@@ -1330,6 +1333,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) pconv_t
                         }
                     }
                 }
+                note_unheld();
             }
 #pragma unroll
             for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
