@@ -20,10 +20,10 @@
 // truncation takes away on average is put back into the weights (tensor_bias).
 // fp16 inputs are exact and need two products.
 //
-// Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 202,
-// 512->512 14x14 183 -> 71, 64->64 224x224 with the pool 547 -> 328, 256->256 28x28 stride 2
+// Measured against pconv_tm (us, batch 32 or 64, keep 0.3; fp32): 256->256 56x56 517 -> 201,
+// 512->512 14x14 183 -> 70, 64->64 224x224 with the pool 547 -> 326, 256->256 28x28 stride 2
 // 200 -> 55; fp16 256->256 28x28 keep 1 808 -> 75.  What bounds it: the MMA rate and the last wave
-// (56x56: 5.36 waves of CTA pairs run as 6; 72 % of the tensor pipe) on the 56x56 and 28x28 layers of
+// (56x56: 5.36 waves of CTA pairs run as 6; 73 % of the tensor pipe) on the 56x56 and 28x28 layers of
 // 256 and 512 filters, the input staging (six warps: split into pairs, store) with 64 filters or
 // stride 2, one partial wave on the smallest.
 #include <cuda.h>
@@ -980,9 +980,9 @@ __device__ __forceinline__ bool unheld(const TcParams& p, const Unit& U, const f
 // image), so that a tap is one offset for all positions; a lane lists the kernels of one channel and
 // group, a slot at a time, with their offsets, and all lanes apply the list.  us a call, keep 0.3, fp32:
 //                              ordinary   one infinity   every unit   FFMA kernel
-//   256 -> 256, 56x56, N 32      203          720          2710           517
-//   512 -> 512, 14x14, N 32       71         1200          1250           187
-//   64 -> 64, 224x224, N 32, pool 328         610          4860           553
+//   256 -> 256, 56x56, N 32      201          720          2710           517
+//   512 -> 512, 14x14, N 32       70         1200          1250           187
+//   64 -> 64, 224x224, N 32, pool 326         610          4860           553
 // (from global memory 6600 and 34900, 21600 and 22000, 4000 and 99000).  The loads of shared memory and
 // the two warps a scheduler bound it.
 template <int S, typename T, int MT>
